@@ -53,11 +53,11 @@
 #include "walk64.cuh"
 
 #define SG_BWD_MAX_W 4
-// lanes of a warp that must be idle before the re-walk refills them together (swept under the
-// length order with the paired grad_V reductions: 16 0.706, 20 0.686, 24 0.648, 28 0.631,
-// 32 0.633 ms)
+// Service threshold and crossings between looks at the lanes' states (run_walks) of the re-walk, 1M
+// queries with grad_V / 262k short walks without: 28 lanes 1 step 616 / 116 us, 24 and 2 609 / 115,
+// 20 and 2 607 / 114, 20 and 3 608 / 114
 #ifndef SG_REWALK_REFILL
-#define SG_REWALK_REFILL 28
+#define SG_REWALK_REFILL 20
 #endif
 // minimum resident blocks per SM the assemble and literal kernels are compiled for (the assemble
 // pass holds no walk since its chord walks moved to a second pass)
@@ -69,14 +69,11 @@
 #ifndef SG_LITERAL_MINB
 #define SG_LITERAL_MINB 7
 #endif
-// walk steps between the re-walk's and the literal walks' refill checks (re-walk: 1 step 0.600 ms,
-// 2 steps 0.619, 3 steps 0.651; refill at 28 idle lanes with one step: 20 0.665, 24 0.619,
-// 30 0.601, 32 0.610 ms; the forward walk keeps 2: 0.389 ms against 0.522 with one)
 #ifndef SG_REWALK_STEPS
-#define SG_REWALK_STEPS 1
+#define SG_REWALK_STEPS 3
 #endif
 #ifndef SG_LITERAL_STEPS
-#define SG_LITERAL_STEPS 2
+#define SG_LITERAL_STEPS 4
 #endif
 // minimum resident blocks per SM of the re-walk (69 registers at 7 without spills, with the
 // straddle test's rare constants, the query id and the face offset in shared memory; 6 blocks
@@ -84,9 +81,10 @@
 #ifndef SG_REWALK_MINB
 #define SG_REWALK_MINB 7
 #endif
-// the same for the literal GFD walks
+// service threshold and steps of the literal GFD walks (the headline's tasks: 24 lanes 2 steps 133 us,
+// 16 and 2 126, 16 and 4 121, 12 and 3 123, 20 and 3 126)
 #ifndef SG_LITERAL_REFILL
-#define SG_LITERAL_REFILL 24
+#define SG_LITERAL_REFILL 16
 #endif
 
 struct BwdArgs {
@@ -384,29 +382,44 @@ struct RewalkHook {
 };
 
 // ------------------------------------------------------------------ kernel 1: re-walk
+// Appends query q's swept columns (bits 0..2 of split) to a task list: one atomic for the calling
+// lanes together, the tasks of one kind next to each other (a literal walk's kind decides its code).
+__device__ __forceinline__ void append_tasks(unsigned split, int32_t q, int32_t *list, int32_t *count) {
+    const unsigned act = __activemask(), below = (1u << (threadIdx.x & 31)) - 1u;
+    const unsigned b0 = __ballot_sync(act, split & 1u), b1 = __ballot_sync(act, split & 2u), b2 = __ballot_sync(act, split & 4u);
+    const int n0 = __popc(b0), n1 = __popc(b1), n = n0 + n1 + __popc(b2);
+    if (n == 0) return;
+    const int leader = __ffs(act) - 1;
+    int base = 0;
+    if ((int)(threadIdx.x & 31) == leader) base = atomicAdd(count, n);
+    base = __shfl_sync(act, base, leader);
+    if (split & 1u) list[base + __popc(b0 & below)] = (q << 2) | 1;
+    if (split & 2u) list[base + n0 + __popc(b1 & below)] = (q << 2) | 2;
+    if (split & 4u) list[base + n0 + n1 + __popc(b2 & below)] = (q << 2) | 3;
+}
+
 template <bool GFD, bool GRADV>
 struct RewalkJob {
     const BwdArgs *A;
     Walker w;
     RewalkHook<GFD, GRADV> H;
-    bool valid;
 
-    __device__ __forceinline__ bool init(int64_t t) {
+    __device__ __forceinline__ int init(int64_t t) {
         // the query (nq < 2^29, checked at the entry point); an order entry out of range (a
         // caller's order that is not a permutation) is skipped
         const int32_t q = A->perm ? __ldg(A->perm + t) : (int32_t)t;
         if ((uint32_t)q >= (uint32_t)A->nq) {
-            s_rewalk_q[threadIdx.x] = -1;
-            valid = false;
-            return false;
+            return SG_LANE_FREE;
         }
         s_rewalk_q[threadIdx.x] = q;
         H.A = A;
         const WalkParams &P = A->P;
         Carry<0> cw;
         bool live = walker_init<0>(P, A->in, q, w, cw);
-        valid = live && !(w.st & SG_ST_INVALID);
-        if (!valid) return false;
+        if (!live || (w.st & SG_ST_INVALID)) {
+            if (A->out_status) A->out_status[q] = (w.st & ~SG_PARITY_BIT) | (GRADV ? SG_ST_NO_GRADV : 0u);
+            return SG_LANE_FREE;
+        }
         s_rewalk_foff[threadIdx.x] = w.foff;
         uint32_t fst = A->end_status ? __ldg(A->end_status + q) : 0u;
         H.gradv = GRADV && !(fst & (SG_ST_VERTEX_HIT | SG_ST_BOUNDARY | SG_ST_MAX_STEPS | SG_ST_INVALID | SG_ST_HOLE));
@@ -456,16 +469,13 @@ struct RewalkJob {
             atomic_add3(A->gacc, fv0.y, b1 * G0 + t1);
             atomic_add3(A->gacc, fv0.z, b2 * G0 + t2);
         }
-        return true;
+        return SG_LANE_SLOW;
     }
-    __device__ __forceinline__ bool step() { return walker_step<true>(w, A->P, H); }
-    __device__ __forceinline__ void finish() {
+    __device__ __forceinline__ int fast() { return fast_step<false, false>(w, A->P, H); }
+    __device__ __forceinline__ int slow() { return walker_step<true>(w, A->P, H) ? SG_LANE_END : walker_ready(w); }
+    __device__ __forceinline__ int end() {
         const int32_t q = s_rewalk_q[threadIdx.x];
-        if (q < 0) return;
-        if (!valid) {
-            if (A->out_status) A->out_status[q] = (w.st & ~SG_PARITY_BIT) | (GRADV ? SG_ST_NO_GRADV : 0u);
-            return;
-        }
+        walker_settle(w, A->P);
         uint32_t st = w.st & ~SG_PARITY_BIT;
         if (GRADV && H.gradv) {
             H.G.flush(A->wacc, w.h);
@@ -496,13 +506,12 @@ struct RewalkJob {
             if (split && !mixed && !(H.S.split & SG_SPLIT_RESTART)) A->rst[2 * (int64_t)q] = make_int4(-1, 0, 0, 0);
             if (split) {
                 st |= SG_ST_GFD_SPLIT;
-                int32_t *list = mixed ? A->tasks40 : A->tasks;
-                int base = atomicAdd(A->ntask + (mixed ? 4 : 0), __popc(split));
-                for (int k = 0; k < 3; ++k)
-                    if (split & (1u << k)) list[base++] = (int32_t)((q << 2) | (k + 1));
             }
+            append_tasks(mixed ? 0u : split, q, A->tasks, A->ntask);
+            append_tasks(mixed ? split : 0u, q, A->tasks40, A->ntask + 4);
         }
         if (A->out_status) A->out_status[q] = st;
+        return SG_LANE_FREE;
     }
 };
 
@@ -510,7 +519,7 @@ template <bool GFD, bool GRADV>
 __global__ void __launch_bounds__(128, SG_REWALK_MINB) k_bwd_rewalk(BwdArgs A) {
     RewalkJob<GFD, GRADV> job;
     job.A = &A;
-    run_persistent<RewalkJob<GFD, GRADV>, SG_REWALK_REFILL, SG_REWALK_STEPS>(A.ntask + 1, A.nq, job);
+    run_walks<RewalkJob<GFD, GRADV>, SG_REWALK_REFILL, SG_REWALK_STEPS>(A.ntask + 1, A.nq, job);
 }
 
 // ------------------------------------------------------------------ chord / literal walks
@@ -640,7 +649,7 @@ struct LiteralJob {
         return true;
     }
 
-    __device__ __forceinline__ bool init(int64_t t) {
+    __device__ __forceinline__ int init(int64_t t) {
         const int32_t task = A->tasks[t];
         q = task >> 2;
         k = task & 3;
@@ -649,7 +658,7 @@ struct LiteralJob {
         L = w.Lh; d0x = w.dx; d0y = w.dy;
         if (restart(k)) {
             phase = 1;
-            return true;
+            return SG_LANE_LIVE;
         }
         if (k == 1) {
             float vx = L * d0x - A->eps_v * d0y, vy = L * d0y + A->eps_v * d0x;
@@ -662,18 +671,23 @@ struct LiteralJob {
             w.dx = ux; w.dy = uy; w.Lh = A->eps_p; w.Ll = 0.f; w.mode = 6;
             phase = 0;
         }
-        return true;
+        return SG_LANE_SLOW;
     }
-    __device__ __forceinline__ bool step() {
-        if (!walker_step<true, HOLE>(w, A->P)) return false;
-        if (phase == 1) return true;
+    __device__ __forceinline__ int fast() { NoHook h; return fast_step<false, false>(w, A->P, h); }
+    __device__ __forceinline__ int slow() { return walker_step<true, HOLE>(w, A->P) ? SG_LANE_END : walker_ready(w); }
+    __device__ __forceinline__ int end() {
+        walker_settle(w, A->P);
+        if (phase == 1) {
+            finish();
+            return SG_LANE_FREE;
+        }
         // end of p -> p_u: continue with v transported along the short walk
         float vc = d0x * ux + d0y * uy, vs = ux * d0y - uy * d0x;  // v/L relative to e_u
         float s_t = (w.st & SG_PARITY_BIT) ? -1.f : 1.f;
         float nx = vc * w.dx - s_t * vs * w.dy, ny = vc * w.dy + s_t * vs * w.dx;
         w.dx = nx; w.dy = ny; w.Lh = L; w.Ll = 0.f; w.mode = 6; w.steps = 0;
         phase = 1;
-        return false;
+        return SG_LANE_SLOW;
     }
     __device__ __forceinline__ void finish() {
         // the forward's end state (the task's own walker supplies the per-query fields)
@@ -690,7 +704,7 @@ template <bool HOLE>
 __global__ void __launch_bounds__(128, SG_LITERAL_MINB) k_bwd_literal(BwdArgs A) {
     LiteralJob<HOLE> job;
     job.A = &A;
-    run_persistent<LiteralJob<HOLE>, SG_LITERAL_REFILL, SG_LITERAL_STEPS>(A.ntask + 2, (int64_t)*A.ntask, job);
+    run_walks<LiteralJob<HOLE>, SG_LITERAL_REFILL, SG_LITERAL_STEPS>(A.ntask + 2, (int64_t)*A.ntask, job);
 }
 
 // The literal walks of the swept columns of a query whose forward walk was the mixed walk (a walk

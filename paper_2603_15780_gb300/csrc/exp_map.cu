@@ -22,19 +22,35 @@
 #include "walk.cuh"
 
 #define SG_MAX_W 4
-// lanes of a warp that must be idle before the forward walk refills them together (walk on 1M
-// queries of the 81,920-face sphere, length order, 256-bit record loads: 8 lanes 0.412 ms, 12
-// 0.403, 16 0.424, 20 0.432)
-// walk steps between refill checks of the forward walk (one: 0.522 ms against 0.389 ms with two)
-// and of the trace
+// Service threshold (lanes of a warp that wait for an end, a start or a rare step before the warp
+// serves them together) and crossings between looks at the lanes' states, per kernel (run_walks).
+// Forward walk, 1M queries on the 81,920-face sphere, length order: 2 steps 337 us, 3 331, 4 329,
+// 6 330; threshold 10 335, 12 329, 14 330, 20 355 us.
 #ifndef SG_WALK_STEPS
-#define SG_WALK_STEPS 2
-#endif
-#ifndef SG_TRACE_STEPS
-#define SG_TRACE_STEPS 2
+#define SG_WALK_STEPS 4
 #endif
 #ifndef SG_WALK_REFILL
 #define SG_WALK_REFILL 12
+#endif
+// trace (10k queries): 2 steps at 12 lanes 51.0 us, 3 at 16 49.1, 4 at 20 49.4
+#ifndef SG_TRACE_STEPS
+#define SG_TRACE_STEPS 3
+#endif
+#ifndef SG_TRACE_REFILL
+#define SG_TRACE_REFILL 16
+#endif
+// mixed walk (4M torus queries / 524k long heightfield walks): 2 steps at 12 lanes 3.79 / 8.89 ms,
+// 3 at 10 3.59 / 8.82, 4 at 8 3.59 / 8.64, 4 at 6 3.69 / 8.43, 6 at 8 3.79 / 8.53
+#ifndef SG_MIX_STEPS
+#define SG_MIX_STEPS 4
+#endif
+#ifndef SG_MIX_REFILL
+#define SG_MIX_REFILL 8
+#endif
+// the hole-avoidance walk keeps the older driver (run_persistent), whose boundary events wait for
+// each other (SG_HOLE_BATCH): on run_walks it took 0.98-1.11 ms against 0.72 ms on 262k queries
+#ifndef SG_HOLE_REFILL
+#define SG_HOLE_REFILL 12
 #endif
 // lanes of a warp with a pending hole-avoidance boundary event before those events run together
 #ifndef SG_HOLE_BATCH
@@ -122,8 +138,9 @@ __global__ void __launch_bounds__(256) k_walk_plain(FwdArgs a) {
                 escalate(a, q);
                 continue;
             }
-            while (!walker_step<ESC>(w, a.P)) {
+            while (!walker_advance<ESC>(w, a.P)) {
             }
+            walker_settle(w, a.P);
             // the step cap of an AUTO walk is its crossing budget (see FwdJob)
             if (AUTO && a.esc_ncross && (w.st & SG_ST_MAX_STEPS)) {
                 escalate(a, q);
@@ -139,43 +156,39 @@ __global__ void __launch_bounds__(256) k_walk_plain(FwdArgs a) {
 // budget is the walk's step cap (P.max_steps, set to it by the host; a crossing is a step, so no
 // walk kept here crosses more edges than that), which costs no test of its own per step; a walk
 // stopped by it is handed on (esc_ncross != 0) unless the caller's own cap is that low.
-template <int NW, bool ESC, bool HOLE = false, bool AUTO = false>
+template <int NW, bool ESC, bool AUTO = false>
 struct FwdJob {
     const FwdArgs *a;
     Walker w;
     Carry<NW> cw;
     int64_t q;
-    __device__ __forceinline__ bool init(int64_t t) {
+    __device__ __forceinline__ int init(int64_t t) {
         q = a->perm ? (int64_t)__ldg(a->perm + t) : t;
-        return walker_init<NW>(a->P, a->in, q, w, cw);
+        if (walker_init<NW>(a->P, a->in, q, w, cw)) return SG_LANE_SLOW;
+        return end();
     }
-    __device__ __forceinline__ bool step() {
-        if (HOLE) {
-            // boundary events of hole avoidance wait until several lanes have one (or every
-            // stepping lane does), then run together
-            const bool pend = w.mode >= SG_MODE_HOLE_EDGE;
-            const unsigned act = __activemask();
-            const unsigned pm = __ballot_sync(act, pend);
-            if (pend && __popc(pm) < SG_HOLE_BATCH && pm != act) return false;
-        }
-        return walker_step<ESC, HOLE>(w, a->P);
+    __device__ __forceinline__ int fast() { NoHook h; return fast_step<false, false>(w, a->P, h); }
+    __device__ __forceinline__ int slow() {
+        return walker_step<ESC>(w, a->P) ? SG_LANE_END : walker_ready(w);
     }
-    __device__ __forceinline__ void finish() {
+    __device__ __forceinline__ int end() {
+        walker_settle(w, a->P);
         if (AUTO && a->esc_ncross && (w.st & SG_ST_MAX_STEPS)) {
             // (one atomic per such query: these are the walks that outran their predicted
             // length, and an aggregated append here costs the walk registers)
             a->esc_list[atomicAdd(a->esc_count, 1)] = (int32_t)q;
-            return;
+            return SG_LANE_FREE;
         }
         walker_finish<NW>(*a, q, w, cw);
+        return SG_LANE_FREE;
     }
 };
 
 template <int NW, bool ESC, bool AUTO = false>
 __global__ void __launch_bounds__(256, 4) k_walk_persistent(FwdArgs a) {
-    FwdJob<NW, ESC, false, AUTO> job;
+    FwdJob<NW, ESC, AUTO> job;
     job.a = &a;
-    run_persistent<FwdJob<NW, ESC, false, AUTO>, SG_WALK_REFILL, SG_WALK_STEPS>(a.counter, a.nq, job);
+    run_walks<FwdJob<NW, ESC, AUTO>, SG_WALK_REFILL, SG_WALK_STEPS>(a.counter, a.nq, job);
 }
 
 // The mixed walk (precision 40; walk.cuh, MIX): the FP32 walker with the direction in
@@ -187,27 +200,28 @@ struct MixJob {
     Walker w;
     Carry<NW> cw;
     int64_t q, n1;
-    __device__ __forceinline__ bool init(int64_t t) {
+    __device__ __forceinline__ int init(int64_t t) {
         if (a->mix_lists) q = t < n1 ? (int64_t)__ldg(a->perm + t) : (int64_t)__ldg(a->esc_list + (t - n1));
         else q = a->perm ? (int64_t)__ldg(a->perm + t) : t;
         w.dxl = 0.f; w.dyl = 0.f;
-        const bool live = walker_init<NW>(a->P, a->in, q, w, cw);
-        if (live) walker_start_mix(a->P, a->in, q, w);
-        return live;
+        if (!walker_init<NW>(a->P, a->in, q, w, cw)) return end();
+        walker_start_mix(a->P, a->in, q, w);
+        return walker_ready(w);
     }
-    __device__ __forceinline__ bool step() { return walker_step<ESC, false, true>(w, a->P); }
-    __device__ __forceinline__ void finish() {
+    __device__ __forceinline__ int fast() { NoHook h; return fast_step<true, false>(w, a->P, h); }
+    __device__ __forceinline__ int slow() {
+        return walker_step<ESC, false, true>(w, a->P) ? SG_LANE_END : walker_ready(w);
+    }
+    __device__ __forceinline__ int end() {
+        walker_settle<true>(w, a->P);
         w.st |= SG_ST_MIXED;
         walker_finish<NW>(*a, q, w, cw);
+        return SG_LANE_FREE;
     }
 };
 
 #ifndef SG_MIX_MINB
 #define SG_MIX_MINB 4
-#endif
-// walk steps between the mixed walk's refill checks (64-mesh batch: 2 steps 17.2 ms, 1 step 17.8 ms)
-#ifndef SG_MIX_STEPS
-#define SG_MIX_STEPS 2
 #endif
 template <int NW, bool ESC>
 __global__ void __launch_bounds__(256, SG_MIX_MINB) k_walk_mixed(FwdArgs a) {
@@ -219,7 +233,7 @@ __global__ void __launch_bounds__(256, SG_MIX_MINB) k_walk_mixed(FwdArgs a) {
         job.n1 = a.route_n ? __ldg(a.route_n) : 0;
         n = job.n1 + __ldg(a.esc_count);
     }
-    run_persistent<MixJob<NW, ESC>, SG_WALK_REFILL, SG_MIX_STEPS>(a.counter, n, job);
+    run_walks<MixJob<NW, ESC>, SG_MIX_REFILL, SG_MIX_STEPS>(a.counter, n, job);
 }
 
 // hole avoidance (boundary_mode 1): the boundary handling needs more registers than the
@@ -234,10 +248,31 @@ __global__ void __launch_bounds__(256, SG_MIX_MINB) k_walk_mixed(FwdArgs a) {
 #define SG_HOLE_STEPS 1
 #endif
 template <int NW>
+struct HoleJob {
+    const FwdArgs *a;
+    Walker w;
+    Carry<NW> cw;
+    int64_t q;
+    __device__ __forceinline__ bool init(int64_t t) {
+        q = a->perm ? (int64_t)__ldg(a->perm + t) : t;
+        return walker_init<NW>(a->P, a->in, q, w, cw);
+    }
+    __device__ __forceinline__ bool step() {
+        // boundary events of hole avoidance wait until several lanes have one (or every
+        // stepping lane does), then run together
+        const bool pend = w.mode >= SG_MODE_HOLE_EDGE;
+        const unsigned act = __activemask();
+        const unsigned pm = __ballot_sync(act, pend);
+        if (pend && __popc(pm) < SG_HOLE_BATCH && pm != act) return false;
+        return walker_step<true, true>(w, a->P);
+    }
+    __device__ __forceinline__ void finish() { walker_finish<NW>(*a, q, w, cw); }
+};
+template <int NW>
 __global__ void __launch_bounds__(256, SG_HOLE_MINB) k_walk_hole(FwdArgs a) {
-    FwdJob<NW, true, true> job;
+    HoleJob<NW> job;
     job.a = &a;
-    run_persistent<FwdJob<NW, true, true>, SG_WALK_REFILL, SG_HOLE_STEPS>(a.counter, a.nq, job);
+    run_persistent<HoleJob<NW>, SG_HOLE_REFILL, SG_HOLE_STEPS>(a.counter, a.nq, job);
 }
 
 // ------------------------------------------------------------------ geodesic tracing
@@ -316,34 +351,41 @@ struct TraceJob {
         }
         n++;
     }
-    __device__ __forceinline__ bool init(int64_t tk) {
+    // the face just entered: by a crossing (the half-edge mode does not keep w.f up to date; px is
+    // the fraction along local edge k from its corner k), or with the walker on a corner
+    __device__ __forceinline__ void rec_crossing() {
+        w.f = w.h / 3;
+        rec(w.px, w.h - 3 * w.f);
+    }
+    __device__ __forceinline__ int init(int64_t tk) {
         q = a->perm ? (int64_t)__ldg(a->perm + tk) : tk;
         n = 0;
-        const bool live = walker_init<0>(a->P, a->in, q, w, cw);
-        if (live && w.Lh > 0.f) rec(0.f, 3);  // Exp_p(0) = p enters no face
-        return live;
+        if (!walker_init<0>(a->P, a->in, q, w, cw)) return end();
+        if (w.Lh > 0.f) rec(0.f, 3);  // Exp_p(0) = p enters no face
+        return SG_LANE_SLOW;
     }
-    __device__ __forceinline__ bool step() {
+    __device__ __forceinline__ int fast() {
+        NoHook h;
+        const int r = fast_step<false, false>(w, a->P, h);
+        if (r == SG_FAST_CROSSED) rec_crossing();
+        return r;
+    }
+    __device__ __forceinline__ int slow() {
         const int nc = w.ncross;
         const bool done = walker_step<ESC>(w, a->P);
-        if (w.ncross != nc) {
-            // entered face h / 3 through its local edge k at fraction px from corner k (in the
-            // half-edge mode the walker does not keep w.f up to date)
-            if (w.mode == SG_MODE_HALF) w.f = w.h / 3;
-            rec(w.px, w.h - 3 * w.f);
-        } else if (!done && w.mode >= 3 && w.mode < 6) {
-            // a vertex transport left the walker on corner mode-3 of face w.f
-            rec(0.f, w.mode - 3);
-        }
-        return done;
+        if (w.ncross != nc) rec_crossing();
+        else if (!done && w.mode >= 3 && w.mode < 6) rec(0.f, w.mode - 3);  // after a vertex transport
+        return done ? SG_LANE_END : walker_ready(w);
     }
-    __device__ __forceinline__ void finish() {
+    __device__ __forceinline__ int end() {
+        walker_settle(w, a->P);
         walker_finish<0>(*a, q, w, cw);
         t->len[q] = n;
         if (t->staged) {  // entries still in the stage
             const int m = min(n, t->cap), rem = m & (SG_TRACE_STAGE - 1), tid = threadIdx.x;
             for (int j = 0; j < rem; ++j) put(q * t->cap + (m - rem) + j, sg->face[j][tid], sg->a[j][tid], sg->code[j][tid]);
         }
+        return SG_LANE_FREE;
     }
 };
 
@@ -393,7 +435,7 @@ __global__ void __launch_bounds__(256, 4) k_trace_persistent(FwdArgs a, TraceOut
     job.a = &a;
     job.t = &t;
     job.sg = &stage;
-    run_persistent<TraceJob<ESC>, SG_WALK_REFILL, SG_TRACE_STEPS>(a.counter, a.nq, job);
+    run_walks<TraceJob<ESC>, SG_TRACE_REFILL, SG_TRACE_STEPS>(a.counter, a.nq, job);
 }
 
 // ------------------------------------------------------------------ start-face counting sort

@@ -132,7 +132,7 @@ struct StepsJob {
         return true;
     }
 
-    __device__ __forceinline__ bool init(int64_t t) {
+    __device__ __forceinline__ int init(int64_t t) {
         q = a->perm ? (int64_t)__ldg(a->perm + t) : t;
         k = 0;
         st_all = 0;
@@ -163,20 +163,26 @@ struct StepsJob {
                 a->step_v[3 * q] = 0.f; a->step_v[3 * q + 1] = 0.f; a->step_v[3 * q + 2] = 0.f;
             }
             end_step();
-            return false;
+            finish();
+            return SG_LANE_FREE;
         }
         const float rs = 1.f / sb;
         b1 = fmaxf(b1, 0.f) * rs; b2 = fmaxf(b2, 0.f) * rs;
         w.px = fmaf(b1, w.R.l01, b2 * w.R.x2x);
         w.py = b2 * w.R.x2y;
-        if (begin_step()) return true;
-        return !end_step();
+        if (begin_step() || !end_step()) return SG_LANE_SLOW;
+        finish();
+        return SG_LANE_FREE;
     }
-    // one step of the current walk; true when it has ended (the driver then calls next())
-    __device__ __forceinline__ bool step() { return walker_step<true>(w, a->P); }
-    // after a walk ended: its records and the next step's start; true when a walk is live again,
-    // false when the query's last step has ended
-    __device__ __forceinline__ bool next() { return !end_step(); }
+    __device__ __forceinline__ int fast() { NoHook h; return fast_step<false, false>(w, a->P, h); }
+    __device__ __forceinline__ int slow() { return walker_step<true>(w, a->P) ? SG_LANE_END : walker_ready(w); }
+    // a walk has ended: its records and the next step's start, or the query's outputs
+    __device__ __forceinline__ int end() {
+        walker_settle(w, a->P);
+        if (!end_step()) return SG_LANE_SLOW;
+        finish();
+        return SG_LANE_FREE;
+    }
     __device__ __forceinline__ void finish() {
         const WalkParams &P = a->P;
         float b0, b1, b2;
@@ -199,60 +205,19 @@ struct StepsJob {
     }
 };
 
-// The persistent driver of walk.cuh (run_persistent), extended by the step transitions: a lane
-// whose walk ended waits, like a lane waiting for a new query, until enough lanes of its warp are
-// idle, and then the waiting lanes start their next steps together (the start interpolates the
-// field and reads the face's axes: a chain of dependent loads that lanes taking it one by one
-// would serialise over the warp).  Once the queue is empty the waiting lanes go on at once.
-#define SG_STEPS_REFILL 12
-// walk steps between refill checks (K = 5, 1M queries: one 1.47 ms, two 1.51 ms)
+// service threshold and crossings between looks at the lanes' states (run_walks; K = 5, 262k
+// queries, 13 crossings a step): 12 lanes 2 steps 387 us, 16 and 2 343, 16 and 4 291, 20 and 4 285,
+// 20 and 6 267 us
+#ifndef SG_STEPS_REFILL
+#define SG_STEPS_REFILL 20
+#endif
 #ifndef SG_KSTEP_STEPS
-#define SG_KSTEP_STEPS 1
+#define SG_KSTEP_STEPS 6
 #endif
 __global__ void __launch_bounds__(256, 4) k_walk_steps(StepsArgs a) {
     StepsJob job;
     job.a = &a;
-    const unsigned FULL = 0xffffffffu;
-    bool live = false, cont = false, pending = false, exhausted = false;
-    while (true) {
-        const unsigned idle = __ballot_sync(FULL, !live);
-        const unsigned waiting = __ballot_sync(FULL, cont);
-        if (exhausted && idle == FULL && !waiting) break;
-        if (__popc(idle) >= SG_STEPS_REFILL || (exhausted && waiting)) {
-            bool dry = false;
-            if (!live) {
-                if (cont) {
-                    cont = false;
-                    live = job.next();
-                    pending = !live;
-                } else if (!exhausted) {
-                    if (pending) {
-                        job.finish();
-                        pending = false;
-                    }
-                    const int64_t t = fetch_ticket(a.counter);
-                    if (t >= a.nq) {
-                        dry = true;
-                    } else {
-                        live = job.init(t);
-                        if (!live) job.finish();
-                    }
-                }
-            }
-            exhausted = exhausted || __any_sync(FULL, dry);
-        }
-#pragma unroll
-        for (int s = 0; s < SG_KSTEP_STEPS; ++s) {
-            if (live && job.step()) {
-                live = false;
-                cont = true;
-            }
-        }
-        if (exhausted && pending) {
-            job.finish();
-            pending = false;
-        }
-    }
+    run_walks<StepsJob, SG_STEPS_REFILL, SG_KSTEP_STEPS>(a.counter, a.nq, job);
 }
 
 // The field's term of step k's VJP (see the file comment), one thread per query: gb_next[q] =

@@ -591,6 +591,22 @@ __device__ __forceinline__ void half_to_face(Walker &w, const WalkParams &P, flo
     w.mode = 6;
 }
 
+// The end of a walk whose length runs out before the exit edge: the final truncated in-face
+// segment (reading: stop once the length is used up), from the half-edge frame into the face frame.
+template <bool MIX = false>
+__device__ __forceinline__ void half_final(Walker &w, const WalkParams &P) {
+    const float near = P.tau_near * w.lref;
+    const float x = w.px * (MIX ? __int_as_float(w.R.n0) : hl(w.R)), L = w.Lh + w.Ll;
+    const float xe = fmaf(L, w.dx, x), ye = L * w.dy;
+    w.Lh = 0.f; w.Ll = 0.f;
+    half_to_face<MIX>(w, P, xe, ye);
+    const FaceRec &F = w.R;
+    float d0 = fabsf(w.py);
+    float d1 = fabsf((F.x2x - F.l01) * (w.py) - F.x2y * (w.px - F.l01)) * F.il1;
+    float d2 = fabsf(F.x2x * w.py - F.x2y * w.px) * F.il2;
+    if (fminf(fminf(d0, d1), d2) <= near) w.st |= SG_ST_NEAR_EDGE;
+}
+
 // The hot step: the walker sits on the entry edge A=(0,0) -> B=(l,0) of half-edge h at
 // x = s*l, the apex is C=(cx,cy) with cy > 0.  sigma_A = dy x, sigma_B = -dy (l - x),
 // sigma_C = dx cy - dy (cx - x).  The exit edge is B -> C when the apex lies left of the ray
@@ -649,15 +665,7 @@ __device__ __forceinline__ bool half_step(Walker &w, const WalkParams &P, Hook &
     const float t = fmaxf(fmaf(qx - x, w.dx, qy * w.dy), 0.f);
     const float L = w.Lh + w.Ll;
     if (t >= L) {
-        // final truncated in-face segment (reading: stop once the length is used up)
-        const float xe = fmaf(L, w.dx, x), ye = L * w.dy;
-        w.Lh = 0.f; w.Ll = 0.f;
-        half_to_face<MIX>(w, P, xe, ye);
-        const FaceRec &F = w.R;
-        float d0 = fabsf(w.py);
-        float d1 = fabsf((F.x2x - F.l01) * (w.py) - F.x2y * (w.px - F.l01)) * F.il1;
-        float d2 = fabsf(F.x2x * w.py - F.x2y * w.px) * F.il2;
-        if (fminf(fminf(d0, d1), d2) <= near) w.st |= SG_ST_NEAR_EDGE;
+        half_final<MIX>(w, P);
         return true;
     }
     {   // compensated L -= t: t < Lh + Ll here, so |Lh| >= |t| up to the tiny Ll and Dekker's
@@ -726,6 +734,85 @@ __device__ __forceinline__ bool half_step(Walker &w, const WalkParams &P, Hook &
     return false;
 }
 
+// The hot step again, as the walk kernels run it: one straight line for the ordinary crossing and
+// one branch for everything else.  All of half_step's tests (another mode than the half-edge one,
+// the step cap, an apex in the near band, a boundary edge) are formed first and taken together;
+// a step that fails one of them changes nothing and is left to walker_step.  A walk whose length
+// ends in this face is only marked: it keeps its half-edge state, and half_final runs when the
+// driver finishes the walks of several lanes together, instead of once per walk for one lane of
+// the warp.  The arithmetic is half_step's, operation for operation.
+#define SG_FAST_CROSSED 0   // the values of SG_LANE_LIVE, _END and _SLOW
+#define SG_FAST_END 1
+#define SG_FAST_SLOW 2
+template <bool MIX, bool ANYMODE, class Hook>
+__device__ __forceinline__ int fast_step(Walker &w, const WalkParams &P, Hook &hook) {
+    const FaceRec &R = w.R;
+    const float near = P.tau_near * w.lref;
+    const float L0 = MIX ? __int_as_float(R.n0) : hl(R);
+    const float cx = MIX ? __int_as_float(R.n2) : hcx(R);
+    const float cy = MIX ? R.x2x : hcy(R);
+    const float x = w.px * L0;
+    const float sA = w.dy * x;
+    const float sB = -w.dy * (L0 - x);
+    const float sC = fmaf(w.dx, cy, -w.dy * (cx - x));
+    const bool right = sC > 0.f;
+    const float x0 = right ? L0 : cx, y0 = right ? 0.f : cy;
+    const float x1 = right ? cx : 0.f, y1 = right ? cy : 0.f;
+    const float s0 = right ? sB : sC, s1 = right ? sC : sA;
+    const float den = s0 - s1;
+    const float s = __saturatef(den != 0.f ? __fdividef(s0, den) : 0.5f);
+    const float qx = fmaf(s, x1 - x0, x0), qy = fmaf(s, y1 - y0, y0);
+    const float t = fmaxf(fmaf(qx - x, w.dx, qy * w.dy), 0.f);
+    const bool end = t >= w.Lh + w.Ll;
+    const int link = MIX ? (right ? __float_as_int(R.il1) : __float_as_int(R.il2)) : (right ? hlinkR(R) : hlinkL(R));
+    if ((ANYMODE && w.mode != SG_MODE_HALF) || w.steps >= P.max_steps || fabsf(sC) < near || (link < 0 && !end))
+        return SG_FAST_SLOW;
+    hook.on_apex(w, sC, cx, cy, x, 0.f);
+    if (end) return SG_FAST_END;
+    const int hn = link >> 1, fl = link & 1;
+    const FaceRec G = load_rec<true>(MIX ? P.half48 : P.half, hn);
+    {   // compensated L -= t (see half_step)
+        const float sum = w.Lh - t;
+        w.Ll += -t - (sum - w.Lh);
+        w.Lh = sum;
+    }
+    float ndx, ndy, re, eda = 0.f, edc = 0.f;
+    if (MIX) {
+        const DF Ld{L0, __int_as_float(R.n1)}, cxd{cx, R.l01}, cyd{cy, R.x2y};
+        const DF dxd{w.dx, w.dxl}, dyd{w.dy, w.dyl};
+        const DF ex = right ? df_sub(cxd, Ld) : df_neg(cxd), ey = right ? cyd : df_neg(cyd);
+        const DF da = df_dot2(dxd, ex, dyd, ey);
+        const DF dc = df_dot2(dxd, ey, df_neg(dyd), ex);
+        re = rsqrtf(fmaf(da.hi, da.hi, dc.hi * dc.hi));
+        const DF nx = df_mul_f(fl ? da : df_neg(da), re), ny = df_mul_f(dc, re);
+        ndx = nx.hi; ndy = ny.hi;
+        w.dxl = nx.lo; w.dyl = ny.lo;
+    } else {
+        const float ex = x1 - x0, ey = y1 - y0;
+        const float da = fmaf(w.dx, ex, w.dy * ey);
+        const float dc = fmaf(w.dx, ey, -w.dy * ex);
+        re = rsqrtf(fmaf(da, da, dc * dc));
+        ndx = (fl ? da : -da) * re; ndy = dc * re;
+        eda = da; edc = dc;
+    }
+    w.steps++;
+    if (!MIX) {
+        const int k = w.h - 3 * (w.h / 3);
+        const int g = hn / 3;
+        hook.on_cross(w, Cross{right ? nxt(k) : prv(k), x0, y0, x1, y1, qx, qy, w.Lh + w.Ll, g, hn - 3 * g, fl,
+                               0.f, 0.f, hl(G), 0.f, ndx, ndy, hca(R), hsa(R), hca(G), hsa(G), re, k, s, eda, edc},
+                      G);
+    }
+    w.px = fl ? s : 1.f - s;
+    w.dx = ndx; w.dy = ndy;
+    w.h = hn;
+    w.R = G;
+    w.st ^= (uint32_t)fl << 31;
+    w.ncross++;
+    if (P.want_hash) walker_hash(w, hn / 3, 1);
+    return SG_FAST_CROSSED;
+}
+
 template <bool ESC, bool HOLE, bool MIX, class Hook>
 __device__ __forceinline__ bool general_step(Walker &w, const WalkParams &P, Hook &hook);
 
@@ -742,6 +829,21 @@ __device__ __forceinline__ bool walker_step(Walker &w, const WalkParams &P, Hook
     w.steps++;
     if (w.mode == SG_MODE_HALF) return half_step<ESC, HOLE, MIX>(w, P, hook);
     return general_step<ESC, HOLE, MIX>(w, P, hook);
+}
+
+// One step of a walk kernel.  Returns true when the walk is finished, except for half_final, which
+// the caller owes a walk that ended in the half-edge mode (walker_settle, before its end is read).
+template <bool ESC, bool HOLE = false, bool MIX = false, class Hook = NoHook>
+__device__ __forceinline__ bool walker_advance(Walker &w, const WalkParams &P, Hook &&hook = Hook()) {
+    const int r = fast_step<MIX, true>(w, P, hook);
+    return r == SG_FAST_SLOW ? walker_step<ESC, HOLE, MIX>(w, P, hook) : r == SG_FAST_END;
+}
+// the lane state of a walk that is about to take a step: an ordinary crossing is possible from the
+// half-edge mode only
+__device__ __forceinline__ int walker_ready(const Walker &w) { return w.mode == SG_MODE_HALF ? 0 : 2; }
+template <bool MIX = false>
+__device__ __forceinline__ void walker_settle(Walker &w, const WalkParams &P) {
+    if (w.mode == SG_MODE_HALF) half_final<MIX>(w, P);
 }
 
 // Step from a corner (after a vertex transport) or from a free start point (face frame); a
@@ -1101,6 +1203,54 @@ __device__ __forceinline__ int64_t fetch_ticket(int32_t *counter) {
     if (lane == leader) base = atomicAdd(counter, __popc(mask));
     base = __shfl_sync(mask, base, leader);
     return (int64_t)base + rank;
+}
+
+// State of a lane of run_walks.
+#define SG_LANE_LIVE 0   // walking
+#define SG_LANE_END 1    // its walk has ended (half_final possibly still owed): job.end() is due
+#define SG_LANE_SLOW 2   // its next step is not an ordinary crossing: job.slow() is due
+#define SG_LANE_FREE 3   // no task
+
+// The walk kernels' driver.  Lanes pull task indices t < n from *counter.  The warp alternates
+// between a hot loop, in which its live lanes take ordinary crossings (fast_step) and nothing else,
+// and a service phase for the lanes that dropped out of it: a walk that ended, a step that is not
+// an ordinary crossing, a lane without a task.  The service phase runs once REFILL lanes of the
+// warp wait for it (each kernel sets its own threshold), so that the long code of an end, a start
+// or a rare step runs with many lanes active, and the hot loop is a loop of its own to the register
+// allocator and the instruction cache.  Once the counter passes n, or when every task got a lane at
+// the start (20k queries: waiting for company took the re-walk from 44 to 57 us), no lane waits for
+// company.
+// Job: int init(t), end(), slow(), each returning the lane's new state (init and end write the
+// outputs of a task that is done); int fast() returns SG_FAST_*.  STEPS crossings run
+// between looks at the lanes' states.
+template <class Job, int REFILL, int STEPS>
+__device__ __forceinline__ void run_walks(int32_t *counter, int64_t n, Job &job) {
+    if (n <= 0) return;  // an empty list (a count read from device memory): no ticket to take
+    const unsigned FULL = 0xffffffffu;
+    // a grid with a lane for every task: the first ticket is a lane's only one
+    const bool once = (int64_t)gridDim.x * blockDim.x >= n;
+    int st = SG_LANE_FREE;
+    bool exhausted = false;
+    for (;;) {
+        if (st == SG_LANE_END) st = job.end();
+        bool dry = false;
+        if (st == SG_LANE_FREE && !exhausted) {
+            const int64_t t = fetch_ticket(counter);
+            if (t < n) st = job.init(t);
+            else dry = true;
+        }
+        exhausted = exhausted || once || __any_sync(FULL, dry);
+        if (st == SG_LANE_SLOW) st = job.slow();
+        if (exhausted && !__any_sync(FULL, st != SG_LANE_FREE)) break;
+        const int wait = exhausted ? 1 : REFILL;
+        unsigned idle;
+        do {
+#pragma unroll
+            for (int k = 0; k < STEPS; ++k)
+                if (st == SG_LANE_LIVE) st = job.fast();
+            idle = __ballot_sync(FULL, st != SG_LANE_LIVE && !(exhausted && st == SG_LANE_FREE));
+        } while (__popc(idle) < wait);
+    }
 }
 
 // Lanes pull task indices t < n from *counter.  A lane whose task has ended keeps its state

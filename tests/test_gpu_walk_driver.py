@@ -1,0 +1,60 @@
+"""The persistent walks (hot loop and service phase) against the one-thread-per-query kernel.
+
+Both run the same steps in the same arithmetic, so every output is equal bit for bit, whatever lanes
+a query shares its warp with: batches around a warp, a block and a full grid, and with starts on
+edges and vertices, invalid queries, zero lengths, boundary stops and low step caps among them.
+"""
+import numpy as np
+import pytest
+
+import meshgen
+
+pytestmark = pytest.mark.gpu
+
+
+def _mesh_and_queries(n, seed):
+    rng = np.random.Generator(np.random.PCG64(seed))
+    X, F, waves = meshgen.heightfield(40, rng)
+    X = meshgen.jitter_slivers(X, 40, rng, 0.10, waves)
+    q = meshgen.sample_queries(X, F, n, rng, 0.0, 0.8, 1)
+    k = np.arange(n)
+    q.bary[k % 11 == 3] = [0.25, 0.75, 0.0]          # on an edge
+    q.bary[k % 13 == 4] = [1.0, 0.0, 0.0]            # on a vertex (half of them point out of the face)
+    q.v[k % 17 == 5] = 0.0
+    q.face[k % 19 == 6] = len(F)                     # no such face
+    q.v[k % 23 == 7] *= np.nan
+    return X, F, q
+
+
+@pytest.mark.parametrize("max_steps", [0, 5])
+@pytest.mark.parametrize("n", [1, 31, 33, 257, 5000])
+def test_persistent_equals_plain(n, max_steps):
+    import torch
+
+    import paper_2603_15780_gb300 as sg
+    X, F, q = _mesh_and_queries(n, 11 + n)
+    mesh = sg.Mesh(X.astype(np.float32), F)
+    args = (mesh, q.face, q.bary.astype(np.float32), q.v.astype(np.float32), q.w.astype(np.float32))
+    kw = {"want_hash": True, "precision": 32, "max_steps": max_steps or None}
+    a = sg.exp_map(*args, **kw)                                        # small batch: one thread per query
+    b = sg.exp_map(*args, kernel=sg.KERNEL_PERSISTENT, **kw)
+    c = sg.exp_map(*args, kernel=sg.KERNEL_PERSISTENT, queries_per_thread=8, block=32, blocks_per_sm=1, sort=2, **kw)
+    torch.cuda.synchronize()
+    for o in (b, c):
+        for k in ("face", "bary", "pos", "dir", "w", "status", "ncross", "hash"):
+            assert torch.equal(a[k].view(torch.uint8), o[k].view(torch.uint8)), k
+
+
+def test_grid_takes_many_tasks_per_lane():
+    """Each lane takes many queries in turn (the first ticket is not a lane's only one)."""
+    import torch
+
+    import paper_2603_15780_gb300 as sg
+    X, F, q = _mesh_and_queries(40000, 5)
+    mesh = sg.Mesh(X.astype(np.float32), F)
+    args = (mesh, q.face, q.bary.astype(np.float32), q.v.astype(np.float32), q.w.astype(np.float32))
+    a = sg.exp_map(*args, want_hash=True, precision=32)
+    b = sg.exp_map(*args, want_hash=True, precision=32, kernel=sg.KERNEL_PERSISTENT, block=32, blocks_per_sm=1)
+    torch.cuda.synchronize()
+    for k in ("face", "bary", "pos", "dir", "w", "status", "ncross", "hash"):
+        assert torch.equal(a[k].view(torch.uint8), b[k].view(torch.uint8)), k
