@@ -673,14 +673,21 @@ struct LiteralJob {
         }
         return SG_LANE_SLOW;
     }
-    __device__ __forceinline__ int fast() { NoHook h; return fast_step<false, false>(w, A->P, h); }
-    __device__ __forceinline__ int slow() { return walker_step<true, HOLE>(w, A->P) ? SG_LANE_END : walker_ready(w); }
-    __device__ __forceinline__ int end() {
-        walker_settle(w, A->P);
-        if (phase == 1) {
-            finish();
-            return SG_LANE_FREE;
+    // the end of the short walk p -> p_u is served like a rare step, before the walk goes on
+    __device__ __forceinline__ int fast() {
+        NoHook h;
+        const int r = fast_step<false, false>(w, A->P, h);
+        if (r != SG_FAST_END || phase == 1) return r;
+        phase = 2;
+        return SG_LANE_SLOW;
+    }
+    __device__ __forceinline__ int slow() {
+        if (phase != 2) {
+            const bool done = walker_step<true, HOLE>(w, A->P);
+            if (!done) return walker_ready(w);
+            if (phase == 1) return SG_LANE_END;
         }
+        walker_settle(w, A->P);
         // end of p -> p_u: continue with v transported along the short walk
         float vc = d0x * ux + d0y * uy, vs = ux * d0y - uy * d0x;  // v/L relative to e_u
         float s_t = (w.st & SG_PARITY_BIT) ? -1.f : 1.f;
@@ -688,6 +695,11 @@ struct LiteralJob {
         w.dx = nx; w.dy = ny; w.Lh = L; w.Ll = 0.f; w.mode = 6; w.steps = 0;
         phase = 1;
         return SG_LANE_SLOW;
+    }
+    __device__ __forceinline__ int end() {
+        walker_settle(w, A->P);
+        finish();
+        return SG_LANE_FREE;
     }
     __device__ __forceinline__ void finish() {
         // the forward's end state (the task's own walker supplies the per-query fields)
@@ -724,7 +736,7 @@ struct Literal40Job {
     __device__ __forceinline__ void to_face() {
         if (w.mode == SG48_END) leave48(w, A->P4, dunpack(w.px), dunpack(w.py), dunpack(w.dx), dunpack(w.dy));
     }
-    __device__ __forceinline__ bool init(int64_t t) {
+    __device__ __forceinline__ int init(int64_t t) {
         const P64 &P = A->P4;
         const QueryIn &in = A->in;
         const int32_t task = A->tasks40[t];
@@ -733,9 +745,9 @@ struct Literal40Job {
         const int m = in.mesh_id ? __ldg(in.mesh_id + q) : 0;
         w.foff = __ldg(P.face_off + m);
         w.f = w.foff + __ldg(in.face + q);
-        w.lref = (double)__ldg(P.lref + m);
-        w.nearf = (float)(P.tau_near * w.lref);
-        w.snapf = (float)(P.tau_snap * w.lref);
+        const double lref = (double)__ldg(P.lref + m);
+        w.near = P.tau_near * lref; w.snap = P.tau_snap * lref;
+        w.nearf = (float)w.near; w.snapf = (float)w.snap;
         w.R = load64(P, w.f);
         double b0 = __ldg(in.bary + 3 * q), b1 = __ldg(in.bary + 3 * q + 1), b2 = __ldg(in.bary + 3 * q + 2);
         const double sb = b0 + b1 + b2;
@@ -759,11 +771,17 @@ struct Literal40Job {
             w.dx = ux; w.dy = uy; w.L = A->eps_p;
             phase = 0;
         }
-        return true;
+        return SG_LANE_LIVE;
     }
-    __device__ __forceinline__ bool step() {
-        if (!step40<0>(w, A->P4)) return false;
-        if (phase == 1) return true;
+    __device__ __forceinline__ int fast() {
+        if (!step40<0>(w, A->P4)) return SG_LANE_LIVE;
+        return phase == 1 ? SG_LANE_END : SG_LANE_SLOW;
+    }
+    __device__ __forceinline__ int end() {
+        finish();
+        return SG_LANE_FREE;
+    }
+    __device__ __forceinline__ int slow() {
         // end of p -> p_u: continue with v transported along the short walk (its angle to the
         // walking direction kept)
         to_face();
@@ -772,7 +790,7 @@ struct Literal40Job {
         const double nx = vc * w.dx - s_t * vs * w.dy, ny = vc * w.dy + s_t * vs * w.dx;
         w.dx = nx; w.dy = ny; w.L = L; w.mode = 6; w.steps = 0;
         phase = 1;
-        return false;
+        return SG_LANE_LIVE;
     }
     __device__ __forceinline__ void finish() {
         to_face();
@@ -802,44 +820,24 @@ struct Literal40Job {
 __global__ void __launch_bounds__(128, SG_LITERAL40_MINB) k_bwd_literal40(BwdArgs A) {
     Literal40Job job;
     job.A = &A;
-    run_persistent<Literal40Job, SG_LITERAL_REFILL>(A.ntask + 5, (int64_t)A.ntask[4], job);
+    run_walks<Literal40Job, SG_LITERAL_REFILL, 2>(A.ntask + 5, (int64_t)A.ntask[4], job);
 }
 
-// Columns the re-walk found unswept are chords from p' (the par column always is); the swept
-// ones were written by k_bwd_literal.  Then the columns are contracted into the gradients.
-// Without WALK a query whose chord leaves the end face is left for a second pass (false).
-template <bool HOLE, bool WALK>
-__device__ __forceinline__ bool assemble_query(const BwdArgs &A, int64_t q) {
+// The direction (end frame) and length of column k's chord from p': k = 0 along the walking direction,
+// 1 across it, 2 and 3 along e_u and e_v.
+__device__ __forceinline__ float chord_dir(const BwdArgs &A, const Walker &w, const EndAdj &E, int k, float &ux, float &uy) {
+    if (k == 0) { ux = E.dmx; uy = E.dmy; }
+    else if (k == 1) rmap(-w.dy, w.dx, w.dx, w.dy, E, ux, uy);
+    else if (k == 2) rmap(1.f, 0.f, w.dx, w.dy, E, ux, uy);
+    else rmap(w.R.x2x * w.R.il2, w.R.x2y * w.R.il2, w.dx, w.dy, E, ux, uy);
+    return k < 2 ? A.eps_v : A.eps_p;
+}
+
+// Contracts the columns c (par, perp, u, v) of query q, whose start state is w, into its gradients.
+__device__ __forceinline__ void write_gradients(const BwdArgs &A, int64_t q, const Walker &w, bool valid, float4 c) {
     const WalkParams &P = A.P;
-    Walker w;
-    Carry<0> cw;
-    bool live = walker_init<0>(P, A.in, q, w, cw);
     F3 gv = f3(0.f, 0.f, 0.f), gp = gv, gb = gv;
-    if (live && !(w.st & SG_ST_INVALID)) {
-        float4 c = *reinterpret_cast<const float4 *>(A.cols + 4 * q);
-        const unsigned split = __float_as_uint(c.x);
-        bool ok = true;
-        {
-            const float d0x = w.dx, d0y = w.dy;
-            EndAdj E = end_adjoint(A, q, w.foff);
-            Walker we;
-            end_walker(A, q, w, E, we);
-            float ux, uy;
-            c.x = chord_col<HOLE, WALK>(P, we, E, E.dmx, E.dmy, A.eps_v, ok);
-            if (!(split & 1u)) {
-                rmap(-d0y, d0x, d0x, d0y, E, ux, uy);
-                c.y = chord_col<HOLE, WALK>(P, we, E, ux, uy, A.eps_v, ok);
-            }
-            if (!(split & 2u)) {
-                rmap(1.f, 0.f, d0x, d0y, E, ux, uy);
-                c.z = chord_col<HOLE, WALK>(P, we, E, ux, uy, A.eps_p, ok);
-            }
-            if (!(split & 4u)) {
-                rmap(w.R.x2x * w.R.il2, w.R.x2y * w.R.il2, d0x, d0y, E, ux, uy);
-                c.w = chord_col<HOLE, WALK>(P, we, E, ux, uy, A.eps_p, ok);
-            }
-        }
-        if (!WALK && !ok) return false;
+    if (valid) {
         Fr2 F0 = load_frm(P, w.f);
         gv = c.x * lift(F0, w.dx, w.dy) + c.y * lift(F0, -w.dy, w.dx);
         F3 eu = lift(F0, 1.f, 0.f), ev = lift(F0, w.R.x2x * w.R.il2, w.R.x2y * w.R.il2);
@@ -853,23 +851,84 @@ __device__ __forceinline__ bool assemble_query(const BwdArgs &A, int64_t q) {
     if (A.grad_v) st3(A.grad_v, q, gv);
     if (A.grad_p) st3(A.grad_p, q, gp);
     if (A.grad_bary) st3(A.grad_bary, q, gb);
-    return true;
 }
 
-// One thread per query; the few queries with a chord that leaves the end face (a few percent)
-// go to a list for k_bwd_assemble_walk, which keeps the walk's registers out of this kernel.
+// Columns the re-walk found unswept are chords from p' (the par column always is); the swept
+// ones were written by k_bwd_literal.  Then the columns are contracted into the gradients.  One
+// thread per query; the few queries with a chord that leaves the end face (a few percent, more on
+// meshes whose edges are not much longer than the finite-difference step) go to a list for
+// k_bwd_assemble_walk, which keeps the walk's registers out of this kernel.
 template <bool HOLE>
 __global__ void __launch_bounds__(128, SG_ASSEMBLE_MINB) k_bwd_assemble(BwdArgs A) {
     const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= A.nq) return;
-    if (!assemble_query<HOLE, false>(A, q)) A.tasks[atomicAdd(A.ntask + 3, 1)] = (int32_t)q;
+    Walker w;
+    Carry<0> cw;
+    const bool valid = walker_init<0>(A.P, A.in, q, w, cw) && !(w.st & SG_ST_INVALID);
+    float4 c = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (valid) {
+        c = *reinterpret_cast<const float4 *>(A.cols + 4 * q);
+        const unsigned split = __float_as_uint(c.x);
+        bool ok = true;
+        const EndAdj E = end_adjoint(A, q, w.foff);
+        Walker we;
+        end_walker(A, q, w, E, we);
+        float ux, uy, len;
+        len = chord_dir(A, w, E, 0, ux, uy);
+        c.x = chord_col<HOLE, false>(A.P, we, E, ux, uy, len, ok);
+        if (!(split & 1u)) {
+            len = chord_dir(A, w, E, 1, ux, uy);
+            c.y = chord_col<HOLE, false>(A.P, we, E, ux, uy, len, ok);
+        }
+        if (!(split & 2u)) {
+            len = chord_dir(A, w, E, 2, ux, uy);
+            c.z = chord_col<HOLE, false>(A.P, we, E, ux, uy, len, ok);
+        }
+        if (!(split & 4u)) {
+            len = chord_dir(A, w, E, 3, ux, uy);
+            c.w = chord_col<HOLE, false>(A.P, we, E, ux, uy, len, ok);
+        }
+        if (!ok) {
+            A.tasks[atomicAdd(A.ntask + 3, 1)] = (int32_t)q;
+            return;
+        }
+    }
+    write_gradients(A, q, w, valid, c);
 }
 
+// The deferred queries, four lanes each: lane k evaluates column k, so that the up to four chord
+// walks of a query, each a chain of dependent loads, run side by side instead of one after the other
+// (one thread per query: 50 us on 262k queries a quarter of which are deferred, issue 7.6% active; this
+// 28 us, and 36 -> 18 us on 20k).
 template <bool HOLE>
 __global__ void __launch_bounds__(128) k_bwd_assemble_walk(BwdArgs A) {
-    const int n = A.ntask[3];
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-        assemble_query<HOLE, true>(A, A.tasks[i]);
+    const int n = A.ntask[3], lane = threadIdx.x & 31, k = lane & 3;
+    const unsigned group = 0xfu << (lane & 28);
+    for (int i = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 2); i < n; i += (int)((gridDim.x * blockDim.x) >> 2)) {
+        const int64_t q = A.tasks[i];
+        Walker w;
+        Carry<0> cw;
+        walker_init<0>(A.P, A.in, q, w, cw);  // (a deferred query is valid)
+        const float4 c = *reinterpret_cast<const float4 *>(A.cols + 4 * q);
+        const unsigned split = __float_as_uint(c.x);
+        float v = k == 1 ? c.y : (k == 2 ? c.z : c.w);
+        if (k == 0 || !((split >> (k - 1)) & 1u)) {
+            const EndAdj E = end_adjoint(A, q, w.foff);
+            Walker we;
+            end_walker(A, q, w, E, we);
+            float ux, uy;
+            const float len = chord_dir(A, w, E, k, ux, uy);
+            bool ok = true;
+            v = chord_col<HOLE, true>(A.P, we, E, ux, uy, len, ok);
+        }
+        const int l0 = lane & 28;
+        float4 r;
+        r.x = __shfl_sync(group, v, l0);
+        r.y = __shfl_sync(group, v, l0 + 1);
+        r.z = __shfl_sync(group, v, l0 + 2);
+        r.w = __shfl_sync(group, v, l0 + 3);
+        if (k == 0) write_gradients(A, q, w, true, r);
+    }
 }
 
 // ------------------------------------------------------------------ end-barycentric upstream
@@ -1172,7 +1231,7 @@ extern "C" sg_status sg_exp_map_backward(const sg_mesh *m, int32_t estimator, fl
         if (pev) cudaEventRecord(pev[1], s);
         // the literal walks are done with the task list: the assemble pass reuses it for the
         // queries it defers (a chord that leaves the end face), counted in ntask[3]
-        const unsigned gw = persistent_grid(k_bwd_assemble_walk<false>, nq / 16 + 1);
+        const unsigned gw = persistent_grid(k_bwd_assemble_walk<false>, nq / 4 + 1);  // (four lanes a query)
         if (r.boundary_mode) {
             k_bwd_literal<true><<<persistent_grid(k_bwd_literal<true>, 3 * nq), 128, 0, s>>>(A);
             k_bwd_assemble<true><<<g128, 128, 0, s>>>(A);

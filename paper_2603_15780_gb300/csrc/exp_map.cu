@@ -671,8 +671,14 @@ WsLayout ws_layout(int64_t nF, int64_t nq, int sort, bool esc = false, bool orde
 // stay in L2 are gathered as fast in any order (icosphere s6 and torus walks are as fast or
 // faster without the start-face order), but lanes holding walks of similar length idle less.
 #define SG_SORT_MIN_BATCH 65536
+// The FP64 walk takes its queries by walk length from this many on: a warp costs the FP64 pipe its
+// longest lane's steps whatever its other lanes do, and the pipe, not the gathers, bounds the walk.
+#define SG_SORT64_MIN_BATCH 1024
 // below this many queries the automatic kernel choice walks one thread per query
 #define SG_SMALL_BATCH 65536
+#ifndef SG_SMALL_BLOCK
+#define SG_SMALL_BLOCK 256
+#endif
 // The automatic precision (sg_opts.precision = 0) keeps a query in the FP32 walk while its walk
 // stays within the range where the FP32 walk's face sequences were measured equal to the
 // double-precision ones: below 256 crossings, no difference in 3.9M walks over icospheres, a
@@ -704,6 +710,7 @@ sg_opts resolve(const sg_opts *o, int64_t nq, int64_t nF) {
     if (r.tau_near <= 0.f) r.tau_near = 1e-4f;
     if (r.tau_snap <= 0.f) r.tau_snap = fminf(r.precision >= 48 ? 1e-12f : 1e-6f, r.tau_near);
     if (r.kernel == SG_KERNEL_AUTO) r.kernel = SG_KERNEL_PERSISTENT;
+    if (r.sort < 0 && r.precision == 64 && r.kernel != SG_KERNEL_PLAIN && nq >= SG_SORT64_MIN_BATCH) r.sort = 2;
     if (r.sort < 0)
         r.sort = nq < SG_SORT_MIN_BATCH ? 0 : (128 * nF > (int64_t)l2_bytes() / 2 ? 1 : 2);
     if (r.kernel == SG_KERNEL_PLAIN) { r.sort = 0; r.fp64_escalate = 0; }
@@ -1087,7 +1094,10 @@ sg_status sg_exp_map(const sg_mesh *m, int64_t nq, const int32_t *mesh_id, const
     // automatic choice walks it one thread per query with the persistent kernel's arithmetic
     // (FP64 classification kept), without the queue and its counter reset.
     if (auto_kernel && nq < SG_SMALL_BATCH && r.precision == 32 && r.boundary_mode == 0 && r.sort == 0)
+    {
         r.kernel = SG_KERNEL_PLAIN;
+        if (r.block == 256) r.block = SG_SMALL_BLOCK;
+    }
     if (r.boundary_mode && r.kernel == SG_KERNEL_PLAIN) return SG_ERR_UNSUPPORTED;
     if (r.precision >= 40 && (r.boundary_mode || r.kernel == SG_KERNEL_PLAIN)) return SG_ERR_UNSUPPORTED;
     cudaStream_t s = (cudaStream_t)stream;

@@ -52,7 +52,8 @@ struct Job64 {
     double cc[NW > 0 ? NW : 1], cs[NW > 0 ? NW : 1];
     int64_t q;
 
-    __device__ __forceinline__ bool init(int64_t t) {
+    __device__ __forceinline__ int init(int64_t t) { return start(t) ? SG_LANE_LIVE : end(); }
+    __device__ __forceinline__ bool start(int64_t t) {
         q = a->perm ? (int64_t)__ldg(a->perm + t) : t;
         const P64 &P = a->P;
         const QueryIn &in = a->in;
@@ -67,7 +68,7 @@ struct Job64 {
         bad = bad || !(lr > 0.f);
         w.foff = foff;
         w.f = bad ? foff : foff + lf;
-        w.lref = bad ? 1.0 : (double)lr;
+        const double lref = bad ? 1.0 : (double)lr;
         w.R = load64(P, w.f);
         double b0 = __ldg(in.bary + 3 * q), b1 = __ldg(in.bary + 3 * q + 1), b2 = __ldg(in.bary + 3 * q + 2);
         const double sb = b0 + b1 + b2;
@@ -75,8 +76,8 @@ struct Job64 {
         for (int k = 0; k < NW; ++k) { cc[k] = 0.0; cs[k] = 0.0; }
         w.px = w.py = w.dx = w.dy = 0.0; w.L = 0.0;
         if (bad) { w.st |= SG_ST_INVALID; return false; }
-        w.nearf = (float)(P.tau_near * w.lref);
-        w.snapf = (float)(P.tau_snap * w.lref);
+        w.near = P.tau_near * lref; w.snap = P.tau_snap * lref;
+        w.nearf = (float)w.near; w.snapf = (float)w.snap;
         if (DFW) {
             const int r = start48();
             if (r >= 0) return r != 0;
@@ -194,8 +195,13 @@ struct Job64 {
         w.mode = SG48_HALF;
         return 1;
     }
-    __device__ __forceinline__ bool step() {
-        return PREC == 48 ? step48<NW>(w, a->P) : step64<NW>(w, a->P);
+    __device__ __forceinline__ int fast() {
+        return (PREC == 48 ? step48<NW>(w, a->P) : step64<NW>(w, a->P)) ? SG_LANE_END : SG_LANE_LIVE;
+    }
+    __device__ __forceinline__ int slow() { return SG_LANE_LIVE; }  // (every step is one of fast's)
+    __device__ __forceinline__ int end() {
+        finish();
+        return SG_LANE_FREE;
     }
     // The end of a double-float walk that stopped inside a face in the half-edge mode: the
     // outputs (float32) from the double-float end point, with FP32 rotations and frames.
@@ -279,11 +285,21 @@ struct Job64 {
     }
 };
 
+// service thresholds (run_walks)
+#ifndef SG_WALK64_REFILL
+#define SG_WALK64_REFILL 16
+#endif
+#ifndef SG_WALK48_REFILL
+#define SG_WALK48_REFILL 8
+#endif
+#ifndef SG_WALK48_STEPS
+#define SG_WALK48_STEPS 2
+#endif
 template <int NW>
 __global__ void __launch_bounds__(128) k_walk64(Fwd64Args a) {
     Job64<NW> job;
     job.a = &a;
-    run_persistent(a.counter, a.nq, job);
+    run_walks<Job64<NW>, SG_WALK64_REFILL, 1>(a.counter, a.nq, job);
 }
 
 // resident blocks per SM the double-float walk is compiled for (icosphere s6, 1M queries: 4
@@ -295,7 +311,7 @@ template <int NW>
 __global__ void __launch_bounds__(128, SG_WALK48_MINB) k_walk48(Fwd64Args a) {
     Job64<NW, 48> job;
     job.a = &a;
-    run_persistent(a.counter, a.nq, job);
+    run_walks<Job64<NW, 48>, SG_WALK48_REFILL, SG_WALK48_STEPS>(a.counter, a.nq, job);
 }
 
 // Double-float half-edge records from the FP64 face shapes, in the layout of the FP32 half-edge
@@ -344,7 +360,7 @@ __global__ void k_geom64_faces(int64_t nF, const int4 *__restrict__ fv, const fl
     const double l12 = sqrt(d12[0] * d12[0] + d12[1] * d12[1] + d12[2] * d12[2]);
     const double l20 = sqrt(e2[0] * e2[0] + e2[1] * e2[1] + e2[2] * e2[2]);
     double *r = rec64 + 6 * f;
-    r[0] = l01; r[1] = x2x; r[2] = x2y; r[3] = 1.0 / l12; r[4] = 1.0 / l20; r[5] = 0.0;
+    r[0] = l01; r[1] = x2x; r[2] = x2y; r[3] = 1.0 / l12; r[4] = 1.0 / l20; r[5] = 1.0 / l01;
     double *fr = frm64 + 6 * f;
     fr[0] = u[0]; fr[1] = u[1]; fr[2] = u[2]; fr[3] = w[0]; fr[4] = w[1]; fr[5] = w[2];
     const double *X[3] = {x0, x1, x2};
@@ -428,13 +444,16 @@ cudaError_t sg_launch_walk64(const sg_mesh *m, const SgFwdIO &io, int n_w, const
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     auto go = [&](auto kern) {
+        // A batch that leaves SMs idle in blocks of 128 takes blocks of one warp, dealt evenly over the
+        // SMs with the longest walks first: the FP64 units, one per SM partition, bound the walk
+        const int block = io.nq < (int64_t)sms * 128 * 4 ? 32 : 128;
         int per = r.blocks_per_sm;
         if (per <= 0) {
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, 128, 0);
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, block, 0);
             per = std::max(per, 1);
         }
-        const int64_t grid = std::min<int64_t>((int64_t)sms * per, std::max<int64_t>((io.nq + 127) / 128, 1));
-        kern<<<(unsigned)grid, 128, 0, s>>>(a);
+        const int64_t grid = std::min<int64_t>((int64_t)sms * per, std::max<int64_t>((io.nq + block - 1) / block, 1));
+        kern<<<(unsigned)grid, block, 0, s>>>(a);
     };
     if (r.precision == 48) {
         switch (n_w) {

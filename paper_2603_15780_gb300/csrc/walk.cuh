@@ -1217,9 +1217,12 @@ __device__ __forceinline__ int64_t fetch_ticket(int32_t *counter) {
 // an ordinary crossing, a lane without a task.  The service phase runs once REFILL lanes of the
 // warp wait for it (each kernel sets its own threshold), so that the long code of an end, a start
 // or a rare step runs with many lanes active, and the hot loop is a loop of its own to the register
-// allocator and the instruction cache.  Once the counter passes n, or when every task got a lane at
-// the start (20k queries: waiting for company took the re-walk from 44 to 57 us), no lane waits for
-// company.
+// allocator and the instruction cache.  Once the counter has passed n, or when every task got a lane
+// at the start, a rare step is served at once, and ended walks wait until no lane of the warp walks:
+// they have no successor to make room for, and serving them one by one, each a chain of dependent
+// loads, held up the lanes still walking (20k queries: re-walk 47 -> 38 us, literal walks 41 -> 34 us; trace of
+// 10k 49 -> 34 us).  The control is uniform over the warp and every vote is taken by all of its lanes
+// in straight line, none behind a condition.
 // Job: int init(t), end(), slow(), each returning the lane's new state (init and end write the
 // outputs of a task that is done); int fast() returns SG_FAST_*.  STEPS crossings run
 // between looks at the lanes' states.
@@ -1230,26 +1233,29 @@ __device__ __forceinline__ void run_walks(int32_t *counter, int64_t n, Job &job)
     // a grid with a lane for every task: the first ticket is a lane's only one
     const bool once = (int64_t)gridDim.x * blockDim.x >= n;
     int st = SG_LANE_FREE;
-    bool exhausted = false;
+    bool exhausted = false, ends = true;  // the same on every lane; every vote is taken by all lanes
     for (;;) {
-        if (st == SG_LANE_END) st = job.end();
+        if (ends && st == SG_LANE_END) st = job.end();
         bool dry = false;
         if (st == SG_LANE_FREE && !exhausted) {
             const int64_t t = fetch_ticket(counter);
             if (t < n) st = job.init(t);
             else dry = true;
         }
-        exhausted = exhausted || once || __any_sync(FULL, dry);
+        const unsigned dried = __ballot_sync(FULL, dry);
+        exhausted = exhausted || once || dried != 0u;
         if (st == SG_LANE_SLOW) st = job.slow();
-        if (exhausted && !__any_sync(FULL, st != SG_LANE_FREE)) break;
-        const int wait = exhausted ? 1 : REFILL;
-        unsigned idle;
+        const unsigned busy = __ballot_sync(FULL, st != SG_LANE_FREE);
+        if (exhausted && busy == 0u) break;
+        unsigned live, slow;
         do {
 #pragma unroll
             for (int k = 0; k < STEPS; ++k)
                 if (st == SG_LANE_LIVE) st = job.fast();
-            idle = __ballot_sync(FULL, st != SG_LANE_LIVE && !(exhausted && st == SG_LANE_FREE));
-        } while (__popc(idle) < wait);
+            live = __ballot_sync(FULL, st == SG_LANE_LIVE);
+            slow = __ballot_sync(FULL, st == SG_LANE_SLOW);
+        } while (exhausted ? (live != 0u && slow == 0u) : (__popc(live) > 32 - REFILL));
+        ends = !exhausted || (live | slow) == 0u;
     }
 }
 

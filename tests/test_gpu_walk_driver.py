@@ -58,3 +58,45 @@ def test_grid_takes_many_tasks_per_lane():
     torch.cuda.synchronize()
     for k in ("face", "bary", "pos", "dir", "w", "status", "ncross", "hash"):
         assert torch.equal(a[k].view(torch.uint8), b[k].view(torch.uint8)), k
+
+
+@pytest.mark.parametrize("precision", [40, 48, 64])
+@pytest.mark.parametrize("n", [33, 1023, 1024, 1500])
+def test_wide_walks_do_not_depend_on_the_order(n, precision):
+    """The FP64 walk takes batches of 1024 queries and more in length order and in one-warp blocks."""
+    import torch
+
+    import paper_2603_15780_gb300 as sg
+    X, F, q = _mesh_and_queries(n, 3 + n)
+    mesh = sg.Mesh(X.astype(np.float32), F)
+    args = (mesh, q.face, q.bary.astype(np.float32), q.v.astype(np.float32), q.w.astype(np.float32))
+    a = sg.exp_map(*args, want_hash=True, precision=precision, sort=0, blocks_per_sm=1)
+    for kw in ({}, {"sort": 2}, {"sort": 1}):
+        b = sg.exp_map(*args, want_hash=True, precision=precision, **kw)
+        torch.cuda.synchronize()
+        for k in ("face", "bary", "pos", "dir", "w", "status", "ncross", "hash"):
+            assert torch.equal(a[k].view(torch.uint8), b[k].view(torch.uint8)), (k, kw)
+
+
+def test_update_of_a_batch_keeps_each_mesh():
+    """Edge lengths are summed per block: blocks of one mesh, and blocks that meet two."""
+    import torch
+
+    import paper_2603_15780_gb300 as sg
+    rng = np.random.Generator(np.random.PCG64(9))
+    meshes = [meshgen.icosphere(2), meshgen.flat_grid(9), meshgen.icosphere(1), meshgen.torus(20, 11)]
+    for scale in (1.0, 3.0):
+        Vs = [(X * scale * (1 + i)).astype(np.float32) for i, (X, _) in enumerate(meshes)]
+        made = sg.Mesh([(V, F) for V, (_, F) in zip(Vs, meshes)])
+        moved = sg.Mesh([(X.astype(np.float32), F) for X, F in meshes])
+        moved.update_vertices(torch.as_tensor(np.concatenate(Vs), device="cuda"))
+        assert abs(made.info().l_ref_mean - moved.info().l_ref_mean) <= 1e-12 * made.info().l_ref_mean
+        ids = rng.integers(0, len(meshes), 500).astype(np.int32)
+        qs = [meshgen.sample_queries(V.astype(np.float64), F, 500, rng, 0.1, 2.0, 0) for V, (_, F) in zip(Vs, meshes)]
+        pick = lambda f: np.stack([getattr(qs[m], f)[i] for i, m in enumerate(ids)])
+        args = (pick("face").astype(np.int32), pick("bary").astype(np.float32), pick("v").astype(np.float32))
+        a, b = (sg.exp_map(m, *args, mesh_id=ids) for m in (made, moved))
+        torch.cuda.synchronize()
+        assert torch.equal(a["face"], b["face"]) and torch.equal(a["ncross"], b["ncross"])
+        assert torch.equal(a["status"], b["status"])
+        assert torch.allclose(a["pos"], b["pos"], rtol=0, atol=1e-6 * 10)
