@@ -27,6 +27,9 @@ __all__ = ["Mesh", "exp_map", "exp_map_backward", "transport_back", "ExpMap", "E
            "ST_REWALK_DIVERGED",
            "KERNEL_AUTO", "KERNEL_PLAIN", "KERNEL_PERSISTENT", "EST_EP", "EST_GFD", "SgError"]
 
+# batches of fewer queries are walked in input order (the library's automatic choice of an order)
+_ORDER_MIN = 65536
+
 ST_BOUNDARY, ST_MAX_STEPS, ST_NEAR_VERTEX, ST_NEAR_EDGE = 1, 2, 4, 8
 ST_VERTEX_HIT, ST_FP64, ST_START_ON_EDGE, ST_INVALID = 16, 32, 64, 128
 ST_GFD_SPLIT, ST_FLIPPED, ST_NO_GRADV = 256, 512, 1024
@@ -126,30 +129,58 @@ def _check(rc, what):
         raise SgError(f"{what}: {msg} (status {rc})")
 
 
+_defaults = None  # the library's default options, filled in once
+
+
 def default_opts(**kw) -> Opts:
-    o = Opts()
-    lib().sg_opts_default(C.byref(o))
+    global _defaults
+    if _defaults is None:
+        o = Opts()
+        lib().sg_opts_default(C.byref(o))
+        _defaults = bytes(o)
+    o = Opts.from_buffer_copy(_defaults)
     for k, v in kw.items():
         if v is not None:
             setattr(o, k, v)
     return o
 
 
+_torch_module = None
+
+
 def _torch():
-    import torch
-    if not torch.cuda.is_available():
-        raise SgError("a CUDA device is required (the library has no CPU path)")
-    return torch
+    """torch, once a CUDA device was found (asked until there is one: the check reads the environment
+    and took 1.5 us, of about 70 us that a small exp_map call spends on the host, for every tensor)."""
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        if not torch.cuda.is_available():
+            raise SgError("a CUDA device is required (the library has no CPU path)")
+        _torch_module = torch
+    return _torch_module
+
+
+def _raw_stream(stream):
+    """cudaStream_t of `stream`, or of torch's current stream (without building a Stream object: two
+    microseconds of each call)."""
+    if stream is not None:
+        return stream.cuda_stream
+    torch = _torch()
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def _ptr(t):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _dev(t, dtype, shape=None):
-    torch = _torch()
+    """`t` as a contiguous CUDA tensor of `dtype` and `shape`; `t` itself when it is one already."""
     if t is None:
         return None
+    torch = _torch()
+    if isinstance(t, torch.Tensor) and t.is_cuda and t.dtype is dtype and t.is_contiguous() and (
+            shape is None or t.shape == shape):
+        return t
     t = torch.as_tensor(t)
     if t.device.type != "cuda":
         t = t.to("cuda", non_blocking=True)
@@ -290,11 +321,11 @@ def exp_map(mesh: Mesh, face, bary, v, w=None, length=None, mesh_id=None, *, wan
     if workspace is not None:
         o.workspace = workspace.data_ptr()
         o.workspace_bytes = workspace.numel()
-    s = stream if stream is not None else torch.cuda.current_stream()
+    s = _raw_stream(stream)
     rc = lib().sg_exp_map(mesh.handle, nq, _ptr(mesh_id), _ptr(face), _ptr(bary), _ptr(v), _ptr(length), nw,
                           _ptr(w), _ptr(out["face"]), _ptr(out["bary"]), _ptr(out["pos"]), _ptr(out["dir"]),
                           _ptr(out.get("w")), _ptr(out["status"]), _ptr(out.get("ncross")),
-                          _ptr(out.get("hash")), C.byref(o), C.c_void_p(s.cuda_stream))
+                          _ptr(out.get("hash")), C.byref(o), s)
     _check(rc, "sg_exp_map")
     out["_workspace"] = workspace
     return out
@@ -331,12 +362,12 @@ def exp_map_trace(mesh: Mesh, face, bary, v, length=None, mesh_id=None, *, path_
         workspace = torch.empty(workspace_size(mesh, nq, o), dtype=torch.uint8, device=dev)
     o.workspace = workspace.data_ptr()
     o.workspace_bytes = workspace.numel()
-    s = stream if stream is not None else torch.cuda.current_stream()
+    s = _raw_stream(stream)
     rc = lib().sg_exp_map_trace(mesh.handle, nq, _ptr(mesh_id), _ptr(face), _ptr(bary), _ptr(v), _ptr(length),
                                 path_cap, _ptr(out["path_face"]), _ptr(out.get("path_pt")), _ptr(out["path_len"]),
                                 _ptr(out["face"]), _ptr(out["bary"]), _ptr(out["pos"]), _ptr(out["dir"]),
                                 _ptr(out["status"]), _ptr(out["ncross"]), _ptr(out.get("hash")), C.byref(o),
-                                C.c_void_p(s.cuda_stream))
+                                s)
     _check(rc, "sg_exp_map_trace")
     return out
 
@@ -362,7 +393,7 @@ def _order_ptr(order, nq: int):
 def exp_map_backward(mesh: Mesh, estimator, face, bary, v, end_face, end_bary, end_dir, end_status, g_pos,
                      mesh_id=None, *, g_bary=None, g_dir=None, g_w=None, eps_v=1e-4, eps_p=1e-4,
                      want_grad_V=False, grad_V=None, opts: Opts | None = None, workspace=None, stream=None,
-                     order=None):
+                     order=None, _inputs_only=False):
     """sg_exp_map_backward.  estimator: "ep"/"gfd" or EST_*.  Upstream gradients: g_pos (end
     point), optional g_bary (end barycentrics), g_dir (end direction), g_w [nq, n_w, 3] (carried
     vectors).  Returns dict(grad_v, grad_p, grad_bary, grad_w (if g_w), grad_V (if requested;
@@ -387,9 +418,10 @@ def exp_map_backward(mesh: Mesh, estimator, face, bary, v, end_face, end_bary, e
         g_w = g_w.reshape(nq, n_w, 3)
     mesh_id = _dev(mesh_id, torch.int32, (nq,))
     dev = face.device
-    res = {"grad_v": torch.empty(nq, 3, device=dev), "grad_p": torch.empty(nq, 3, device=dev),
-           "grad_bary": torch.empty(nq, 3, device=dev),
-           "status": torch.empty(nq, dtype=torch.int32, device=dev)}
+    res = {"grad_v": torch.empty(nq, 3, device=dev), "grad_bary": torch.empty(nq, 3, device=dev)}
+    if not _inputs_only:  # (the autograd Function reads neither)
+        res["grad_p"] = torch.empty(nq, 3, device=dev)
+        res["status"] = torch.empty(nq, dtype=torch.int32, device=dev)
     if n_w:
         res["grad_w"] = torch.empty(nq, n_w, 3, device=dev)
     if want_grad_V or grad_V is not None:
@@ -404,13 +436,13 @@ def exp_map_backward(mesh: Mesh, estimator, face, bary, v, end_face, end_bary, e
                                 device=dev)
     o.workspace = workspace.data_ptr()
     o.workspace_bytes = workspace.numel()
-    s = stream if stream is not None else torch.cuda.current_stream()
+    s = _raw_stream(stream)
     rc = lib().sg_exp_map_backward(mesh.handle, est, eps_v, eps_p, nq, _ptr(mesh_id), _ptr(face), _ptr(bary),
                                    _ptr(v), _ptr(end_face), _ptr(end_bary), _ptr(end_dir), _ptr(end_status),
                                    _ptr(g_pos), _ptr(g_bary), _ptr(g_dir), n_w, _ptr(g_w if n_w else None),
-                                   _ptr(res["grad_v"]), _ptr(res["grad_p"]), _ptr(res["grad_bary"]),
-                                   _ptr(res.get("grad_V")), _ptr(res.get("grad_w")), _ptr(res["status"]),
-                                   C.byref(o), C.c_void_p(s.cuda_stream))
+                                   _ptr(res["grad_v"]), _ptr(res.get("grad_p")), _ptr(res["grad_bary"]),
+                                   _ptr(res.get("grad_V")), _ptr(res.get("grad_w")), _ptr(res.get("status")),
+                                   C.byref(o), s)
     _check(rc, "sg_exp_map_backward")
     return res
 
@@ -435,10 +467,10 @@ def transport_back(mesh: Mesh, face, bary, v, end, u, mesh_id=None, *, opts: Opt
     mesh_id = _dev(mesh_id, torch.int32, (nq,))
     out = torch.empty(nq, n_u, 3, device=face.device)
     o = opts if opts is not None else default_opts()
-    s = stream if stream is not None else torch.cuda.current_stream()
+    s = _raw_stream(stream)
     rc = lib().sg_transport_back(mesh.handle, nq, _ptr(mesh_id), _ptr(face), _ptr(bary), _ptr(v), _ptr(end_face),
                                  _ptr(end_dir), _ptr(end_status), n_u, _ptr(u), _ptr(out), C.byref(o),
-                                 C.c_void_p(s.cuda_stream))
+                                 s)
     _check(rc, "sg_transport_back")
     return out.reshape(shape)
 
@@ -472,12 +504,12 @@ def exp_map_field_steps(mesh: Mesh, face, bary, U, K: int, h: float | None = Non
     ws = torch.empty(64, dtype=torch.uint8, device=dev)
     o.workspace = ws.data_ptr()
     o.workspace_bytes = 64
-    s = stream if stream is not None else torch.cuda.current_stream()
+    s = _raw_stream(stream)
     rc = lib().sg_exp_map_steps(mesh.handle, K, h, _ptr(U), nq, _ptr(mesh_id), _ptr(face), _ptr(bary),
                                 _ptr(out["face"]), _ptr(out["bary"]), _ptr(out["pos"]), _ptr(out["dir"]),
                                 _ptr(out["status"]), _ptr(out.get("step_face")), _ptr(out.get("step_bary")),
                                 _ptr(out.get("step_v")), _ptr(out.get("step_dir")), _ptr(out.get("step_status")),
-                                _ptr(out.get("step_hash")), C.byref(o), C.c_void_p(s.cuda_stream))
+                                _ptr(out.get("step_hash")), C.byref(o), s)
     _check(rc, "sg_exp_map_steps")
     out["_workspace"] = ws
     return out
@@ -508,12 +540,12 @@ def exp_map_field_steps_backward(mesh: Mesh, estimator, fwd: dict, U, K: int, h:
     o = opts if opts is not None else default_opts()
     o.workspace = ws.data_ptr()
     o.workspace_bytes = ws.numel()
-    s = stream if stream is not None else torch.cuda.current_stream()
+    s = _raw_stream(stream)
     rc = lib().sg_exp_map_steps_backward(mesh.handle, est, eps_v, eps_p, K, h, _ptr(U), nq, _ptr(mesh_id),
                                          _ptr(fwd["step_face"]), _ptr(fwd["step_bary"]), _ptr(fwd["step_v"]),
                                          _ptr(fwd["step_dir"]), _ptr(fwd["step_status"]), _ptr(g_pos), _ptr(g_bary),
                                          _ptr(res["grad_U"]), _ptr(res["grad_bary"]), _ptr(res.get("grad_V")),
-                                         C.byref(o), C.c_void_p(s.cuda_stream))
+                                         C.byref(o), s)
     _check(rc, "sg_exp_map_steps_backward")
     res["_workspace"] = ws
     return res
@@ -530,12 +562,14 @@ def _autograd_function():
 
         @staticmethod
         def forward(ctx, mesh, face, bary, v, estimator="gfd", V=None, mesh_id=None, eps=1e-4):
-            # the forward's query order is kept for the backward's re-walk (no second sort)
-            order = torch.empty(face.numel(), dtype=torch.int32, device=face.device)
-            out = exp_map(mesh, face, bary.detach(), v.detach(), mesh_id=mesh_id, order=order)
+            bary, v = bary.detach(), v.detach()
+            # the forward's query order is kept for the backward's re-walk (no second sort); a batch too
+            # small to be ordered has a lane for every query and gains nothing by one (three launches)
+            order = (torch.empty(face.numel(), dtype=torch.int32, device=face.device)
+                     if face.numel() >= _ORDER_MIN else None)
+            out = exp_map(mesh, face, bary, v, mesh_id=mesh_id, order=order, want_ncross=False)
             ctx.mesh, ctx.estimator, ctx.eps = mesh, estimator, eps
-            ctx.save_for_backward(face, bary.detach(), v.detach(), out["face"], out["bary"], out["dir"],
-                                  out["status"], mesh_id if mesh_id is not None else torch.empty(0), order)
+            ctx.save_for_backward(face, bary, v, out["face"], out["bary"], out["dir"], out["status"], mesh_id, order)
             ctx.has_V = V is not None
             ctx.mark_non_differentiable(out["face"], out["status"])
             ctx.set_materialize_grads(False)
@@ -547,11 +581,10 @@ def _autograd_function():
             if g_pos is None:
                 g_pos = torch.zeros(face.numel(), 3, device=face.device)
             r = exp_map_backward(ctx.mesh, ctx.estimator, face, bary, v, ef, eb, ed, es, g_pos.contiguous(),
-                                 mesh_id=mid if mid.numel() else None,
-                                 g_bary=None if g_bary is None else g_bary.contiguous(),
+                                 mesh_id=mid, g_bary=None if g_bary is None else g_bary.contiguous(),
                                  g_dir=None if g_dir is None else g_dir.contiguous(),
                                  eps_v=ctx.eps, eps_p=ctx.eps,
-                                 want_grad_V=ctx.has_V and ctx.needs_input_grad[5], order=order)
+                                 want_grad_V=ctx.has_V and ctx.needs_input_grad[5], order=order, _inputs_only=True)
             gV = r.get("grad_V")
             return None, None, r["grad_bary"], r["grad_v"], None, gV, None, None
 
@@ -604,7 +637,7 @@ def _steps_autograd_function():
             out = exp_map_field_steps(mesh, face, bary.detach(), U.detach(), K, h, mesh_id=mesh_id)
             ctx.mesh, ctx.K, ctx.h, ctx.estimator, ctx.eps = mesh, K, h, estimator, eps
             ctx.rec = {k: out[k] for k in ("face", "step_face", "step_bary", "step_v", "step_dir", "step_status")}
-            ctx.save_for_backward(U.detach(), mesh_id if mesh_id is not None else torch.empty(0))
+            ctx.save_for_backward(U.detach(), mesh_id)
             ctx.mark_non_differentiable(out["face"], out["status"])
             ctx.set_materialize_grads(False)
             return out["pos"], out["face"], out["bary"], out["dir"], out["status"]
@@ -617,7 +650,7 @@ def _steps_autograd_function():
                 g_pos = torch.zeros(nq, 3, device=U.device)
             r = exp_map_field_steps_backward(ctx.mesh, ctx.estimator, ctx.rec, U, ctx.K, ctx.h, g_pos.contiguous(),
                                              None if g_bary is None else g_bary.contiguous(),
-                                             mesh_id=mid if mid.numel() else None, eps_v=ctx.eps, eps_p=ctx.eps)
+                                             mesh_id=mid, eps_v=ctx.eps, eps_p=ctx.eps)
             return None, None, r["grad_bary"], r["grad_U"], None, None, None, None, None
 
     return ExpMapFieldSteps

@@ -48,6 +48,7 @@
 #include <algorithm>
 #include <cstring>
 
+#include "launch.cuh"
 #include "sgeo_internal.h"
 #include "walk.cuh"
 #include "walk64.cuh"
@@ -1074,14 +1075,10 @@ namespace {
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 // SM-filling grid of 128-thread blocks for a persistent kernel over n tasks
-template <class K>
-unsigned persistent_grid(K kernel, int64_t n) {
-    int dev = 0, sms = 0, per = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, 128, 0);
-    int64_t need = (n + 127) / 128;
-    return (unsigned)std::max<int64_t>(1, std::min<int64_t>((int64_t)sms * std::max(per, 1), need));
+template <auto KERNEL>
+unsigned persistent_grid(int64_t n) {
+    const int64_t need = (n + 127) / 128;
+    return (unsigned)std::max<int64_t>(1, std::min<int64_t>((int64_t)sg_sm_count() * sg_blocks_per_sm<KERNEL>(128), need));
 }
 struct BwdLayout {
     size_t gacc, wacc, cols, tasks, tasks40, rst, ntask, gpos, lcounts, lkeys, perm, total;
@@ -1222,23 +1219,23 @@ extern "C" sg_status sg_exp_map_backward(const sg_mesh *m, int32_t estimator, fl
     if (estimator == SG_EST_EP) {
         k_ep_backward<<<g256, 256, 0, s>>>(A);
         // the grad_V re-walk rewrites the status with its walk's bits and SG_ST_NO_GRADV
-        if (grad_V) k_bwd_rewalk<false, true><<<persistent_grid(k_bwd_rewalk<false, true>, nq), 128, 0, s>>>(A);
+        if (grad_V) k_bwd_rewalk<false, true><<<persistent_grid<k_bwd_rewalk<false, true>>(nq), 128, 0, s>>>(A);
     } else {
         cudaEvent_t *pev = (cudaEvent_t *)r.prof_events;
         if (pev) cudaEventRecord(pev[0], s);
-        if (grad_V) k_bwd_rewalk<true, true><<<persistent_grid(k_bwd_rewalk<true, true>, nq), 128, 0, s>>>(A);
-        else k_bwd_rewalk<true, false><<<persistent_grid(k_bwd_rewalk<true, false>, nq), 128, 0, s>>>(A);
+        if (grad_V) k_bwd_rewalk<true, true><<<persistent_grid<k_bwd_rewalk<true, true>>(nq), 128, 0, s>>>(A);
+        else k_bwd_rewalk<true, false><<<persistent_grid<k_bwd_rewalk<true, false>>(nq), 128, 0, s>>>(A);
         if (pev) cudaEventRecord(pev[1], s);
         // the literal walks are done with the task list: the assemble pass reuses it for the
         // queries it defers (a chord that leaves the end face), counted in ntask[3]
-        const unsigned gw = persistent_grid(k_bwd_assemble_walk<false>, nq / 4 + 1);  // (four lanes a query)
+        const unsigned gw = persistent_grid<k_bwd_assemble_walk<false>>(nq / 4 + 1);  // (four lanes a query)
         if (r.boundary_mode) {
-            k_bwd_literal<true><<<persistent_grid(k_bwd_literal<true>, 3 * nq), 128, 0, s>>>(A);
+            k_bwd_literal<true><<<persistent_grid<k_bwd_literal<true>>(3 * nq), 128, 0, s>>>(A);
             k_bwd_assemble<true><<<g128, 128, 0, s>>>(A);
             k_bwd_assemble_walk<true><<<gw, 128, 0, s>>>(A);
         } else {
-            k_bwd_literal<false><<<persistent_grid(k_bwd_literal<false>, 3 * nq), 128, 0, s>>>(A);
-            k_bwd_literal40<<<persistent_grid(k_bwd_literal40, 3 * nq), 128, 0, s>>>(A);
+            k_bwd_literal<false><<<persistent_grid<k_bwd_literal<false>>(3 * nq), 128, 0, s>>>(A);
+            k_bwd_literal40<<<persistent_grid<k_bwd_literal40>(3 * nq), 128, 0, s>>>(A);
             k_bwd_assemble<false><<<g128, 128, 0, s>>>(A);
             k_bwd_assemble_walk<false><<<gw, 128, 0, s>>>(A);
         }

@@ -18,6 +18,7 @@
 #include <new>
 #include <vector>
 
+#include "launch.cuh"
 #include "sgeo_internal.h"
 #include "walk.cuh"
 
@@ -46,6 +47,10 @@
 #endif
 #ifndef SG_MIX_REFILL
 #define SG_MIX_REFILL 8
+#endif
+// threads per block of a small batch's walk (20k queries: 32 24.8, 64 24.8, 128 24.3, 256 25.5 us)
+#ifndef SG_SMALL_BLOCK
+#define SG_SMALL_BLOCK 128
 #endif
 // the hole-avoidance walk keeps the older driver (run_persistent), whose boundary events wait for
 // each other (SG_HOLE_BATCH): on run_walks it took 0.98-1.11 ms against 0.72 ms on 262k queries
@@ -208,6 +213,14 @@ struct MixJob {
         walker_start_mix(a->P, a->in, q, w);
         return walker_ready(w);
     }
+    // the walk of query qq, known to be valid
+    __device__ __forceinline__ int start(int64_t qq) {
+        q = qq;
+        w.dxl = 0.f; w.dyl = 0.f;
+        walker_init<NW>(a->P, a->in, q, w, cw);
+        walker_start_mix(a->P, a->in, q, w);
+        return walker_ready(w);
+    }
     __device__ __forceinline__ int fast() { NoHook h; return fast_step<true, false>(w, a->P, h); }
     __device__ __forceinline__ int slow() {
         return walker_step<ESC, false, true>(w, a->P) ? SG_LANE_END : walker_ready(w);
@@ -219,6 +232,41 @@ struct MixJob {
         return SG_LANE_FREE;
     }
 };
+
+// A small batch under the automatic choices, one thread per query in one launch: a query that is too
+// long for FP32 from the start, or whose FP32 walk reaches the crossing budget, goes on in the mixed
+// walk in its own thread.  (With the list of such queries and a second kernel for it, the call was a
+// counter reset and two launches, 1.4-1.8 us each on the device and three on the host, most of the
+// time for an empty list.)  Same walks, same results.
+template <int NW>
+__global__ void __launch_bounds__(SG_SMALL_BLOCK) k_walk_small(FwdArgs a, int mix_max_steps) {
+    const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= a.nq) return;
+    {
+        Walker w;
+        Carry<NW> cw;
+        bool mixed = false;
+        if (walker_init<NW>(a.P, a.in, q, w, cw)) {
+            mixed = w.Lh > a.esc_lmax * w.lref;
+            if (!mixed) {
+                while (!walker_advance<true>(w, a.P)) {
+                }
+                walker_settle(w, a.P);
+                mixed = a.esc_ncross && (w.st & SG_ST_MAX_STEPS);
+            }
+        }
+        if (!mixed) {
+            walker_finish<NW>(a, q, w, cw);
+            return;
+        }
+    }
+    a.P.max_steps = mix_max_steps;
+    MixJob<NW, true> job;
+    job.a = &a;
+    int st = job.start(q);
+    while (st != SG_LANE_END) st = st == SG_LANE_LIVE ? job.fast() : job.slow();
+    job.end();
+}
 
 #ifndef SG_MIX_MINB
 #define SG_MIX_MINB 4
@@ -676,9 +724,6 @@ WsLayout ws_layout(int64_t nF, int64_t nq, int sort, bool esc = false, bool orde
 #define SG_SORT64_MIN_BATCH 1024
 // below this many queries the automatic kernel choice walks one thread per query
 #define SG_SMALL_BATCH 65536
-#ifndef SG_SMALL_BLOCK
-#define SG_SMALL_BLOCK 256
-#endif
 // The automatic precision (sg_opts.precision = 0) keeps a query in the FP32 walk while its walk
 // stays within the range where the FP32 walk's face sequences were measured equal to the
 // double-precision ones: below 256 crossings, no difference in 3.9M walks over icospheres, a
@@ -726,22 +771,14 @@ cudaError_t launch_walk(const FwdArgs &a, const sg_opts &o, cudaStream_t s) {
         else k_walk_plain<NW, false, AUTO><<<(unsigned)grid, o.block, 0, s>>>(a);
         return cudaGetLastError();
     }
-    int dev = 0, sms = 0, per = o.blocks_per_sm;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (per <= 0) {
-        if (o.fp64_escalate)
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_walk_persistent<NW, true>, o.block, 0);
-        else
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_walk_persistent<NW, false>, o.block, 0);
-        per = std::max(per, 1);
-    }
+    const int sms = sg_sm_count();
+    int per = o.blocks_per_sm;
+    if (per <= 0)
+        per = o.fp64_escalate ? sg_blocks_per_sm<k_walk_persistent<NW, true>>(o.block)
+                              : sg_blocks_per_sm<k_walk_persistent<NW, false>>(o.block);
     int64_t need = (a.nq + o.block - 1) / o.block;
     if (o.boundary_mode) {  // hole avoidance: its own instantiation, FP64 classification
-        if (o.blocks_per_sm <= 0) {
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_walk_hole<NW>, o.block, 0);
-            per = std::max(per, 1);
-        }
+        if (o.blocks_per_sm <= 0) per = sg_blocks_per_sm<k_walk_hole<NW>>(o.block);
         int64_t grid = std::min<int64_t>((int64_t)sms * per, std::max<int64_t>(need, 1));
         k_walk_hole<NW><<<(unsigned)grid, o.block, 0, s>>>(a);
         return cudaGetLastError();
@@ -759,14 +796,10 @@ cudaError_t launch_walk(const FwdArgs &a, const sg_opts &o, cudaStream_t s) {
 
 template <int NW>
 cudaError_t launch_mixed(const FwdArgs &a, const sg_opts &o, cudaStream_t s) {
-    int dev = 0, sms = 0, per = o.blocks_per_sm;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (per <= 0) {
-        if (o.fp64_escalate) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_walk_mixed<NW, true>, 256, 0);
-        else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_walk_mixed<NW, false>, 256, 0);
-        per = std::max(per, 1);
-    }
+    const int sms = sg_sm_count();
+    int per = o.blocks_per_sm;
+    if (per <= 0)
+        per = o.fp64_escalate ? sg_blocks_per_sm<k_walk_mixed<NW, true>>(256) : sg_blocks_per_sm<k_walk_mixed<NW, false>>(256);
     const int64_t grid = std::min<int64_t>((int64_t)sms * per, std::max<int64_t>((a.nq + 255) / 256, 1));
     if (o.fp64_escalate) k_walk_mixed<NW, true><<<(unsigned)grid, 256, 0, s>>>(a);
     else k_walk_mixed<NW, false><<<(unsigned)grid, 256, 0, s>>>(a);
@@ -1031,9 +1064,7 @@ sg_status prepare_queue(const sg_mesh *m, int64_t nq, const int32_t *mesh_id, co
         int64_t nk = esc ? 2 * m->nF + 1 : m->nF + 1;
         int64_t ntiles = (nk + SCAN_TILE - 1) / SCAN_TILE;
         cudaMemsetAsync(counts, 0, sizeof(int32_t) * nk, s);
-        int dev = 0, sms = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        const int sms = sg_sm_count();
         int g = (int)std::min<int64_t>((nq + 255) / 256, (int64_t)sms * 8);
         k_sort_keys_hist<<<g, 256, 0, s>>>(nq, a.in, m->d_face_off, m->d_srank, m->d_lref, (int32_t)m->nF, lmax, counts);
         k_scan_tiles<<<(unsigned)ntiles, SCAN_BLOCK, 0, s>>>(counts, nk, sums);
@@ -1056,9 +1087,7 @@ sg_status prepare_queue(const sg_mesh *m, int64_t nq, const int32_t *mesh_id, co
 
 void sg_length_order(const sg_mesh *m, const QueryIn &in, int64_t nq, uint8_t *keys, int32_t *counts, int32_t *perm,
                      cudaStream_t s, float esc_lmax) {
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int sms = sg_sm_count();
     cudaMemsetAsync(counts, 0, sizeof(int32_t) * 2 * SG_LBUCKETS, s);
     const int64_t g1 = std::min<int64_t>((nq + 255) / 256, (int64_t)sms * 4);
     k_lorder_hist<<<(unsigned)std::max<int64_t>(g1, 1), 256, 0, s>>>(nq, in, m->d_lref, esc_lmax, keys, counts);
@@ -1094,10 +1123,7 @@ sg_status sg_exp_map(const sg_mesh *m, int64_t nq, const int32_t *mesh_id, const
     // automatic choice walks it one thread per query with the persistent kernel's arithmetic
     // (FP64 classification kept), without the queue and its counter reset.
     if (auto_kernel && nq < SG_SMALL_BATCH && r.precision == 32 && r.boundary_mode == 0 && r.sort == 0)
-    {
         r.kernel = SG_KERNEL_PLAIN;
-        if (r.block == 256) r.block = SG_SMALL_BLOCK;
-    }
     if (r.boundary_mode && r.kernel == SG_KERNEL_PLAIN) return SG_ERR_UNSUPPORTED;
     if (r.precision >= 40 && (r.boundary_mode || r.kernel == SG_KERNEL_PLAIN)) return SG_ERR_UNSUPPORTED;
     cudaStream_t s = (cudaStream_t)stream;
@@ -1107,8 +1133,9 @@ sg_status sg_exp_map(const sg_mesh *m, int64_t nq, const int32_t *mesh_id, const
     a.out_w = out_w; a.out_status = out_status; a.out_ncross = out_ncross; a.out_hash = out_hash;
 
     const bool persistent = r.kernel == SG_KERNEL_PERSISTENT;
+    const bool small = auto_kernel && autoprec && !persistent && r.fp64_escalate && r.queries_per_thread <= 1;
     void *own_ws = nullptr;
-    if (persistent || autoprec || r.order) {
+    if (persistent || (autoprec && !small) || r.order) {
         sg_status st = prepare_queue(m, nq, mesh_id, face, r, persistent ? r.sort : 0, s, a, &own_ws, autoprec);
         if (st != SG_OK) {
             if (own_ws) cudaFreeAsync(own_ws, s);
@@ -1150,14 +1177,24 @@ sg_status sg_exp_map(const sg_mesh *m, int64_t nq, const int32_t *mesh_id, const
     }
     if (pev) cudaEventRecord(pev[0], s);
     cudaError_t e;
-    switch (n_w) {
+    if (small) {
+        const unsigned grid = (unsigned)((nq + SG_SMALL_BLOCK - 1) / SG_SMALL_BLOCK);
+        switch (n_w) {
+            case 0: k_walk_small<0><<<grid, SG_SMALL_BLOCK, 0, s>>>(a, r.max_steps); break;
+            case 1: k_walk_small<1><<<grid, SG_SMALL_BLOCK, 0, s>>>(a, r.max_steps); break;
+            case 2: k_walk_small<2><<<grid, SG_SMALL_BLOCK, 0, s>>>(a, r.max_steps); break;
+            case 3: k_walk_small<3><<<grid, SG_SMALL_BLOCK, 0, s>>>(a, r.max_steps); break;
+            default: k_walk_small<4><<<grid, SG_SMALL_BLOCK, 0, s>>>(a, r.max_steps); break;
+        }
+        e = cudaGetLastError();
+    } else switch (n_w) {
         case 0: e = autoprec ? launch_walk<0, true>(a, r, s) : launch_walk<0>(a, r, s); break;
         case 1: e = autoprec ? launch_walk<1, true>(a, r, s) : launch_walk<1>(a, r, s); break;
         case 2: e = autoprec ? launch_walk<2, true>(a, r, s) : launch_walk<2>(a, r, s); break;
         case 3: e = autoprec ? launch_walk<3, true>(a, r, s) : launch_walk<3>(a, r, s); break;
         default: e = autoprec ? launch_walk<4, true>(a, r, s) : launch_walk<4>(a, r, s); break;
     }
-    if (e == cudaSuccess && autoprec) {
+    if (e == cudaSuccess && autoprec && !small) {
         // the mixed walk takes the queries the order routed to it (in that order), then those the
         // FP32 walk handed on at its crossing budget; its grid reads the lists' lengths from
         // device memory (no host synchronisation)
@@ -1206,15 +1243,11 @@ sg_status sg_exp_map_trace(const sg_mesh *m, int64_t nq, const int32_t *mesh_id,
         if (own_ws) cudaFreeAsync(own_ws, s);
         return st;
     }
-    int dev = 0, sms = 0, per = r.blocks_per_sm;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int sms = sg_sm_count();
+    int per = r.blocks_per_sm;
     const bool esc = r.fp64_escalate && r.kernel != SG_KERNEL_PLAIN;
-    if (per <= 0) {
-        if (esc) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_trace_persistent<true>, r.block, 0);
-        else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_trace_persistent<false>, r.block, 0);
-        per = std::max(per, 1);
-    }
+    if (per <= 0)
+        per = esc ? sg_blocks_per_sm<k_trace_persistent<true>>(r.block) : sg_blocks_per_sm<k_trace_persistent<false>>(r.block);
     int64_t grid = std::min<int64_t>((int64_t)sms * per, std::max<int64_t>((nq + r.block - 1) / r.block, 1));
     if (esc) k_trace_persistent<true><<<(unsigned)grid, r.block, 0, s>>>(a, t);
     else k_trace_persistent<false><<<(unsigned)grid, r.block, 0, s>>>(a, t);

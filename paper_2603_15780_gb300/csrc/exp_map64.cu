@@ -22,6 +22,7 @@
 
 #include <algorithm>
 
+#include "launch.cuh"
 #include "sgeo_internal.h"
 #include "walk.cuh"
 
@@ -440,36 +441,30 @@ cudaError_t sg_launch_walk64(const sg_mesh *m, const SgFwdIO &io, int n_w, const
     a.out_face = io.out_face; a.out_bary = io.out_bary; a.out_pos = io.out_pos; a.out_dir = io.out_dir;
     a.out_w = io.out_w; a.out_status = io.out_status; a.out_ncross = io.out_ncross; a.out_hash = io.out_hash;
     a.perm = io.perm; a.counter = io.counter;
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    auto go = [&](auto kern) {
+    const int sms = sg_sm_count();
+    auto go = [&](auto kern, auto per_sm) {
         // A batch that leaves SMs idle in blocks of 128 takes blocks of one warp, dealt evenly over the
         // SMs with the longest walks first: the FP64 units, one per SM partition, bound the walk
         const int block = io.nq < (int64_t)sms * 128 * 4 ? 32 : 128;
-        int per = r.blocks_per_sm;
-        if (per <= 0) {
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, block, 0);
-            per = std::max(per, 1);
-        }
+        const int per = r.blocks_per_sm > 0 ? r.blocks_per_sm : per_sm(block);
         const int64_t grid = std::min<int64_t>((int64_t)sms * per, std::max<int64_t>((io.nq + block - 1) / block, 1));
         kern<<<(unsigned)grid, block, 0, s>>>(a);
     };
     if (r.precision == 48) {
         switch (n_w) {
-            case 0: go(k_walk48<0>); break;
-            case 1: go(k_walk48<1>); break;
-            case 2: go(k_walk48<2>); break;
-            case 3: go(k_walk48<3>); break;
-            default: go(k_walk48<4>); break;
+            case 0: go(k_walk48<0>, sg_blocks_per_sm<k_walk48<0>>); break;
+            case 1: go(k_walk48<1>, sg_blocks_per_sm<k_walk48<1>>); break;
+            case 2: go(k_walk48<2>, sg_blocks_per_sm<k_walk48<2>>); break;
+            case 3: go(k_walk48<3>, sg_blocks_per_sm<k_walk48<3>>); break;
+            default: go(k_walk48<4>, sg_blocks_per_sm<k_walk48<4>>); break;
         }
     } else {
         switch (n_w) {
-            case 0: go(k_walk64<0>); break;
-            case 1: go(k_walk64<1>); break;
-            case 2: go(k_walk64<2>); break;
-            case 3: go(k_walk64<3>); break;
-            default: go(k_walk64<4>); break;
+            case 0: go(k_walk64<0>, sg_blocks_per_sm<k_walk64<0>>); break;
+            case 1: go(k_walk64<1>, sg_blocks_per_sm<k_walk64<1>>); break;
+            case 2: go(k_walk64<2>, sg_blocks_per_sm<k_walk64<2>>); break;
+            case 3: go(k_walk64<3>, sg_blocks_per_sm<k_walk64<3>>); break;
+            default: go(k_walk64<4>, sg_blocks_per_sm<k_walk64<4>>); break;
         }
     }
     return cudaGetLastError();

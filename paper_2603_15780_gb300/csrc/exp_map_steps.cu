@@ -23,6 +23,7 @@
 
 #include <algorithm>
 
+#include "launch.cuh"
 #include "sgeo_internal.h"
 #include "walk.cuh"
 
@@ -297,12 +298,7 @@ sg_status sg_exp_map_steps(const sg_mesh *m, int32_t K, float h, const float *U,
     }
     a.counter = (int32_t *)ws;
     cudaMemsetAsync(a.counter, 0, 64, s);
-    int dev = 0, sms = 0, per = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_walk_steps, 256, 0);
-    per = std::max(per, 1);
-    const int64_t grid = std::min<int64_t>((int64_t)sms * per, (nq + 255) / 256);
+    const int64_t grid = std::min<int64_t>((int64_t)sg_sm_count() * sg_blocks_per_sm<k_walk_steps>(256), (nq + 255) / 256);
     cudaEvent_t *pev = (cudaEvent_t *)r.prof_events;
     if (pev) cudaEventRecord(pev[0], s);
     k_walk_steps<<<(unsigned)grid, 256, 0, s>>>(a);

@@ -100,3 +100,34 @@ def test_update_of_a_batch_keeps_each_mesh():
         assert torch.equal(a["face"], b["face"]) and torch.equal(a["ncross"], b["ncross"])
         assert torch.equal(a["status"], b["status"])
         assert torch.allclose(a["pos"], b["pos"], rtol=0, atol=1e-6 * 10)
+
+
+@pytest.mark.parametrize("n", [1, 127, 129, 3000])
+@pytest.mark.parametrize("max_steps", [0, 300])
+def test_small_batches_of_the_automatic_precision(n, max_steps):
+    """One launch for a small batch, with the mixed walks in their queries' own threads: each query's
+    outputs are those of the mixed walk where its status says so, else of the FP32 walk -- queries that
+    are too long for FP32 at the start, and (long thin triangles: more crossings per mean edge length)
+    ones that reach the crossing budget."""
+    import torch
+
+    import paper_2603_15780_gb300 as sg
+    X, F = meshgen.torus(200, 8)
+    rng = np.random.Generator(np.random.PCG64(n))
+    q = meshgen.sample_queries(X, F, n, rng, 0.0, 25.0, 2)
+    q.v[np.arange(n) % 7 == 3] *= 0.05
+    mesh = sg.Mesh(X.astype(np.float32), F)
+    args = (mesh, q.face, q.bary.astype(np.float32), q.v.astype(np.float32), q.w.astype(np.float32))
+    kw = {"want_hash": True, "max_steps": max_steps or None}
+    a = sg.exp_map(*args, **kw)
+    fp32 = sg.exp_map(*args, precision=32, **kw)
+    wide = sg.exp_map(*args, precision=40, **kw)
+    torch.cuda.synchronize()
+    mixed = (a["status"] & sg.ST_MIXED) != 0
+    for k in ("face", "bary", "pos", "dir", "w", "status", "ncross", "hash"):
+        m = mixed.reshape(-1, *[1] * (a[k].dim() - 1))
+        assert torch.equal(a[k].view(torch.uint8), torch.where(m, wide[k], fp32[k]).view(torch.uint8)), k
+    long = torch.as_tensor(np.linalg.norm(q.v, axis=1), device="cuda") > 96 * mesh.info().l_ref_mean
+    assert torch.equal(mixed, long | (fp32["ncross"] >= 256))
+    if n == 3000:
+        assert bool((mixed & long).any()) and bool((mixed & ~long).any()) and bool((~mixed).any())
