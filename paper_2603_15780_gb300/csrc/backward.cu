@@ -139,8 +139,9 @@ struct Fr2 {
     float e1x, e1y, e1z, e2x, e2y, e2z;
 };
 __device__ __forceinline__ Fr2 load_frm(const WalkParams &P, int f) {
-    float4 a = __ldg(P.frm + 2 * f), b = __ldg(P.frm + 2 * f + 1);
-    return Fr2{a.x, a.y, a.z, a.w, b.x, b.y};
+    Fr2 F;
+    frm_axes(P, f, F.e1x, F.e1y, F.e1z, F.e2x, F.e2y, F.e2z);
+    return F;
 }
 __device__ __forceinline__ F3 lift(const Fr2 &F, float a, float b) {
     return f3(a * F.e1x + b * F.e2x, a * F.e1y + b * F.e2y, a * F.e1z + b * F.e2z);

@@ -286,8 +286,10 @@ __global__ void __launch_bounds__(256, SG_MIX_MINB) k_walk_mixed(FwdArgs a) {
 
 // hole avoidance (boundary_mode 1): the boundary handling needs more registers than the
 // default walk, so it gets its own kernel and residency bound
+// (3 blocks of 256: 80 registers; at 4, 64 registers, 442 bytes of spills made 57 memory instructions a
+// crossing: 717 us, at 3 529, at 2 613 on 262k queries)
 #ifndef SG_HOLE_MINB
-#define SG_HOLE_MINB 4
+#define SG_HOLE_MINB 3
 #endif
 // walk steps between the hole-avoidance walk's refill checks: one (the boundary handling makes
 // the loop body large; the sphere with 8% of its faces removed, 1M queries: 2.41 ms, against

@@ -31,13 +31,13 @@ struct FaceRec {
     float l01, x2x, x2y, il1, il2;
 };
 
-// One 32-byte record = one L2 sector, read as two 16-byte loads or, with W, as one 256-bit
-// load (sm_100 and later).  The wide load halves the L2 requests per record and doubles the
-// device's dependent-gather ceiling; the half-edge record of every crossing is read with it
-// (1M queries on an 81,920-face sphere, queries in walk-length order: forward walk 0.437 ->
-// 0.404 ms, backward re-walk 0.738 -> 0.716 ms, whose L2 tag lookups had run at 74% with two
-// 16-byte loads and an atomic per crossing).
-template <bool W = false>
+// One 32-byte record = one L2 sector, read with one 256-bit load (sm_100 and later) or, without W, as
+// two 16-byte loads.  The wide load halves the requests per record and doubles the device's
+// dependent-gather ceiling: the half-edge record of every crossing (1M queries on an 81,920-face
+// sphere, queries in walk-length order: forward walk 0.437 -> 0.404 ms, backward re-walk 0.738 -> 0.716
+// ms, whose L2 tag lookups had run at 74% with two 16-byte loads and an atomic per crossing), and the
+// face records and frames that the elementwise kernels gather (k_bwd_assemble 64 -> 57 us on 1M queries).
+template <bool W = true>
 __device__ __forceinline__ void ld_rec32(const int4 *__restrict__ p, int4 &a, int4 &b) {
     if (W) {
         asm("ld.global.nc.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
@@ -49,7 +49,7 @@ __device__ __forceinline__ void ld_rec32(const int4 *__restrict__ p, int4 &a, in
     }
 }
 
-template <bool W = false>
+template <bool W = true>
 __device__ __forceinline__ FaceRec load_rec(const int4 *__restrict__ rec, int f) {
     int4 a, b;
     ld_rec32<W>(rec + 2 * f, a, b);
@@ -251,8 +251,10 @@ __device__ __forceinline__ DF df_dot2(DF a, DF b, DF c, DF d) {
 //   - a decision closer than tau_near is flagged NEAR_VERTEX.
 __device__ __forceinline__ void frm_axes(const WalkParams &P, int f, float &e1x, float &e1y, float &e1z, float &e2x,
                                          float &e2y, float &e2z) {
-    const float4 a = __ldg(P.frm + 2 * f), b = __ldg(P.frm + 2 * f + 1);
-    e1x = a.x; e1y = a.y; e1z = a.z; e2x = a.w; e2y = b.x; e2z = b.y;
+    int4 a, b;
+    ld_rec32(reinterpret_cast<const int4 *>(P.frm + 2 * f), a, b);
+    e1x = __int_as_float(a.x); e1y = __int_as_float(a.y); e1z = __int_as_float(a.z);
+    e2x = __int_as_float(a.w); e2y = __int_as_float(b.x); e2z = __int_as_float(b.y);
 }
 
 // The walker sits on corner c of face w.f (a boundary vertex; w.R is the face record).
