@@ -501,19 +501,40 @@ __device__ __forceinline__ float query_length(const QueryIn &in, int64_t i) {
 // face centroids, offset by the mesh's first face); nF for an invalid query.  With the automatic
 // precision (esc_lmax > 0) the queries longer than esc_lmax l_ref, which the mixed walk takes,
 // keep that rank as key and form the permutation's head; the others get nF + the rank, and an
-// invalid query 2 nF.
+// invalid query 2 nF.  On meshes of SG_FAR_MIN_FACES and more, the head's head are the walks longer than
+// SG_FAR_LREF l_ref, by length (a quarter of an octave per class, longest first), then place (1024 cells):
+// thousands of crossings leave the neighbourhood of the start at once, so starting together gains them
+// little, and one that starts late ends alone.  To make room for their keys the head's other queries
+// share a key in pairs of ranks.  (A 2.1M-face heightfield, 524k queries, the whole call: lengths up to 3,300
+// l_ref 9.16 -> 7.99 ms, up to 1,650 6.38 -> 5.79, up to 1,100 5.17 -> 4.94.  The line: up to 660 l_ref
+// 3.61 ms by place, 3.66 by length first; up to 330, 3.28 against 3.80; up to 55, 0.67 against 0.92.)
+#define SG_FAR_LREF 768.f
+#define SG_FAR_CLASSES 16
+#define SG_FAR_CELLS 1024
+#define SG_FAR_KEYS (SG_FAR_CLASSES * SG_FAR_CELLS)
+#define SG_FAR_MIN_FACES 65536
+// keys of the automatic precision's head: all of the mixed walk's queries sort below this
+__host__ __device__ __forceinline__ int face_head_keys(int32_t nF) {
+    return nF >= SG_FAR_MIN_FACES ? SG_FAR_KEYS + (nF + 1) / 2 : nF;
+}
 __device__ __forceinline__ int face_key(const QueryIn &in, const int32_t *__restrict__ face_off,
                                         const int32_t *__restrict__ srank, const float *__restrict__ lref,
                                         int32_t nF, float esc_lmax, int64_t i) {
-    const int inval = esc_lmax > 0.f ? 2 * nF : nF;
+    const int head = esc_lmax > 0.f ? face_head_keys(nF) : 0, inval = head + nF;
     const int m = in.mesh_id ? __ldg(in.mesh_id + i) : 0;
     if (m < 0 || m >= in.n_mesh) return inval;
     const int lo = __ldg(face_off + m), hi = __ldg(face_off + m + 1);
     const int f = __ldg(in.face + i);
     if (f < 0 || f >= hi - lo) return inval;
-    int key = __ldg(srank + lo + f);  // in [lo, hi): the face's place on the mesh's Z-order curve
-    if (esc_lmax > 0.f && !(query_length(in, i) > esc_lmax * __ldg(lref + m))) key += nF;
-    return key;
+    const int rank = __ldg(srank + lo + f);  // in [lo, hi): the face's place on the mesh's Z-order curve
+    if (!(esc_lmax > 0.f)) return rank;
+    const float L = query_length(in, i), lr = __ldg(lref + m);
+    if (!(L > esc_lmax * lr)) return head + rank;
+    if (nF < SG_FAR_MIN_FACES) return rank;
+    if (!(L > SG_FAR_LREF * lr)) return SG_FAR_KEYS + rank / 2;
+    const int c = (int)fminf(fmaxf(4.f * __log2f(L / (SG_FAR_LREF * lr)), 0.f), (float)(SG_FAR_CLASSES - 1));
+    const int cell = min((int)((float)rank * ((float)SG_FAR_CELLS / (float)nF)), SG_FAR_CELLS - 1);
+    return (SG_FAR_CLASSES - 1 - c) * SG_FAR_CELLS + cell;
 }
 
 __global__ void k_sort_keys_hist(int64_t nq, QueryIn in, const int32_t *__restrict__ face_off,
@@ -523,8 +544,8 @@ __global__ void k_sort_keys_hist(int64_t nq, QueryIn in, const int32_t *__restri
         atomicAdd(counts + face_key(in, face_off, srank, lref, nF, esc_lmax, i), 1);
 }
 
-// after the scatter offsets[k] is the end of bucket k (with the automatic precision offsets[nF - 1]
-// is the number of routed queries at the head)
+// after the scatter offsets[k] is the end of bucket k (with the automatic precision the end of the head's
+// last bucket is the number of routed queries)
 __global__ void k_sort_scatter(int64_t nq, QueryIn in, const int32_t *__restrict__ face_off,
                                const int32_t *__restrict__ srank, const float *__restrict__ lref, int32_t nF,
                                float esc_lmax, int32_t *__restrict__ offsets, int32_t *__restrict__ perm) {
@@ -697,7 +718,7 @@ WsLayout ws_layout(int64_t nF, int64_t nq, int sort, bool esc = false, bool orde
     L.counter = o; o = align_up(o + 64, 256);
     if (esc) { L.esc = o; o = align_up(o + sizeof(int32_t) * std::max<int64_t>(nq, 1), 256); }
     if (sort == 1) {
-        int64_t nk = esc ? 2 * nF + 1 : nF + 1;
+        int64_t nk = (esc ? face_head_keys((int32_t)nF) : 0) + nF + 1;
         int64_t ntiles = (nk + SCAN_TILE - 1) / SCAN_TILE;
         L.counts = o; o = align_up(o + sizeof(int32_t) * nk, 256);
         L.sums = o; o = align_up(o + sizeof(int32_t) * ntiles, 256);
@@ -1063,7 +1084,7 @@ sg_status prepare_queue(const sg_mesh *m, int64_t nq, const int32_t *mesh_id, co
     } else if (sort == 1) {
         int32_t *counts = (int32_t *)(base + L.counts);
         int32_t *sums = (int32_t *)(base + L.sums);
-        int64_t nk = esc ? 2 * m->nF + 1 : m->nF + 1;
+        int64_t nk = (esc ? face_head_keys((int32_t)m->nF) : 0) + m->nF + 1;
         int64_t ntiles = (nk + SCAN_TILE - 1) / SCAN_TILE;
         cudaMemsetAsync(counts, 0, sizeof(int32_t) * nk, s);
         const int sms = sg_sm_count();
@@ -1075,7 +1096,7 @@ sg_status prepare_queue(const sg_mesh *m, int64_t nq, const int32_t *mesh_id, co
         k_sort_scatter<<<g, 256, 0, s>>>(nq, a.in, m->d_face_off, m->d_srank, m->d_lref, (int32_t)m->nF, lmax, counts,
                                          perm);
         a.perm = perm;
-        if (esc) a.route_n = counts + m->nF - 1;  // the head: up to the end of bucket nF - 1
+        if (esc) a.route_n = counts + face_head_keys((int32_t)m->nF) - 1;  // the end of the head's last bucket
     }
     // the FP32 walk starts its tickets after the routed head
     if (a.route_n && cudaMemcpyAsync(a.counter, a.route_n, sizeof(int32_t), cudaMemcpyDeviceToDevice, s) != cudaSuccess)

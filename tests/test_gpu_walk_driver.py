@@ -131,3 +131,64 @@ def test_small_batches_of_the_automatic_precision(n, max_steps):
     assert torch.equal(mixed, long | (fp32["ncross"] >= 256))
     if n == 3000:
         assert bool((mixed & long).any()) and bool((mixed & ~long).any()) and bool((~mixed).any())
+
+
+@pytest.mark.parametrize("n", [150, 182, 183])   # 44,402, 65,522 and 66,248 faces: around the far walks' line
+def test_start_face_order_with_far_walks(n):
+    """Walks of up to 3,000 mean edge lengths: each query's outputs are those of the walk that its status
+    names, wherever the order puts it."""
+    import torch
+
+    import paper_2603_15780_gb300 as sg
+    rng = np.random.Generator(np.random.PCG64(n))
+    X, F = meshgen.torus(n - 1, n - 1) if n > 150 else meshgen.torus(149, 149)
+    q = meshgen.sample_queries(X, F, 3001, rng, 0.0, 1.0, 0)
+    mesh = sg.Mesh(X.astype(np.float32), F)
+    q.v *= (mesh.info().l_ref_mean * 10.0 ** rng.uniform(-1.0, 3.5, 3001))[:, None]
+    q.face[::97] = len(F)
+    args = (mesh, q.face, q.bary.astype(np.float32), q.v.astype(np.float32))
+    a = sg.exp_map(*args, sort=1, kernel=sg.KERNEL_PERSISTENT, want_hash=True)
+    fp32 = sg.exp_map(*args, precision=32, want_hash=True)
+    wide = sg.exp_map(*args, precision=40, want_hash=True)
+    torch.cuda.synchronize()
+    mixed = (a["status"] & sg.ST_MIXED) != 0
+    assert bool(mixed.any()) and not bool(mixed.all())
+    for k in ("face", "bary", "pos", "dir", "status", "ncross", "hash"):
+        m = mixed.reshape(-1, *[1] * (a[k].dim() - 1))
+        assert torch.equal(a[k].view(torch.uint8), torch.where(m, wide[k], fp32[k]).view(torch.uint8)), k
+
+
+def test_field_gradient_with_and_without_the_accumulator():
+    """A workspace without room for the accumulator is still accepted; both ways sum the same terms."""
+    import ctypes as C
+
+    import torch
+
+    import paper_2603_15780_gb300 as sg
+    X, F = meshgen.icosphere(3)
+    rng = np.random.Generator(np.random.PCG64(4))
+    q = meshgen.sample_queries(X, F, 3001, rng, 0.0, 1.0, 0)
+    mesh, K, nq = sg.Mesh(X.astype(np.float32), F), 3, 3001
+    cu = lambda x: torch.as_tensor(np.asarray(x, np.float32), device="cuda")
+    U, g = cu(rng.normal(size=X.shape)), cu(q.g_pos)
+    fwd = sg.exp_map_field_steps(mesh, q.face, q.bary.astype(np.float32), U, K)
+    n = C.c_size_t()
+    assert sg.lib().sg_exp_map_steps_backward_workspace_size(mesh.handle, sg.EST_GFD, K, nq, 0, C.byref(n)) == 0
+    room = (16 * len(X) + 255) // 256 * 256
+    out = []
+    for size in (n.value, n.value - room, n.value - room - 1):
+        ws = torch.empty(size, dtype=torch.uint8, device="cuda")
+        o = sg.default_opts(workspace=ws.data_ptr(), workspace_bytes=size)
+        gU, gb = torch.ones_like(U), torch.empty(nq, 3, device="cuda")
+        p = lambda x: x.data_ptr()
+        rc = sg.lib().sg_exp_map_steps_backward(
+            mesh.handle, sg.EST_GFD, 1e-3, 1e-3, K, 1.0 / K, p(U), nq, None, p(fwd["step_face"]), p(fwd["step_bary"]),
+            p(fwd["step_v"]), p(fwd["step_dir"]), p(fwd["step_status"]), p(g), None, p(gU), p(gb), None, C.byref(o),
+            torch.cuda.current_stream().cuda_stream)
+        torch.cuda.synchronize()
+        out.append((rc, gU.double(), gb))
+    assert [r[0] for r in out] == [0, 0, 5]   # the last: SG_ERR_OOM
+    assert torch.equal(out[0][2], out[1][2])
+    # about 3001 * 3 * 3 / 642 terms a vertex, summed in float32 in another order
+    scale = float(out[1][1].abs().max())
+    assert float((out[0][1] - out[1][1]).abs().max()) <= 64 * 2.0 ** -24 * scale
