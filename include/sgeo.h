@@ -77,9 +77,10 @@ typedef struct sg_opts {
     int32_t max_steps;      /* loop cap per query (Alg. gpu_parallel MAX_STEPS); <= 0: 1<<20 */
     int32_t kernel;         /* SG_KERNEL_*; AUTO: the persistent kernel, except that sg_exp_map
                                walks a batch of fewer than 65,536 queries taken in input order
-                               (FP32 precision, boundary_mode 0) one thread per query with the
-                               persistent kernel's arithmetic (FP64 classification kept): such a
-                               batch fills the persistent grid once, so the queue gains nothing */
+                               (FP32 or automatic precision, boundary_mode 0) one thread per query
+                               with the persistent kernel's arithmetic (FP64 classification kept),
+                               in one launch: such a batch fills the persistent grid once, so the
+                               queue gains nothing */
     int32_t sort;           /* order in which the persistent kernels take the queries:
                                0: input order; 1: by (mesh, start face), the faces taken along
                                the mesh's Z-order curve of face centroids so that neighbouring
@@ -88,7 +89,11 @@ typedef struct sg_opts {
                                bucket: lanes of a warp then finish together and idle less);
                                <0: auto -- for batches of >= 65536 queries, 1 on meshes whose
                                walk records (128 B per face) exceed half of L2 (locality of the
-                               gathers), else 2; input order for smaller batches.  Outputs are
+                               gathers), else 2; input order for smaller batches; precision 64
+                               takes 2 from 1024 queries on (a workspace without room for it
+                               keeps the order of the other precisions).  In order 1, under the
+                               automatic precision and on 65536 faces and more, the walks longer
+                               than 768 l_ref come first, longest first.  Outputs are
                                always in input order.  sg_exp_map_backward's re-walk uses the
                                length order when sort is 2, or auto with >= 65536 queries. */
     int32_t block;          /* threads per block; <= 0: 256 */

@@ -237,15 +237,17 @@ struct MixJob {
 // long for FP32 from the start, or whose FP32 walk reaches the crossing budget, goes on in the mixed
 // walk in its own thread.  (With the list of such queries and a second kernel for it, the call was a
 // counter reset and two launches, 1.4-1.8 us each on the device and three on the host, most of the
-// time for an empty list.)  Same walks, same results.
+// time for an empty list.)  Same walks, same results.  The mixed walks run on the
+// persistent kernels' hot loop (run_lanes): 20k long walks on a 320,000-face sliver heightfield take 797
+// us; 1,446 with a plain loop per thread, 1,183 with the list and the older driver.  The FP32 walks are
+// too short to gain by it and take the plain loop: 24 against 28 us on 20k.
 template <int NW>
 __global__ void __launch_bounds__(SG_SMALL_BLOCK) k_walk_small(FwdArgs a, int mix_max_steps) {
     const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= a.nq) return;
-    {
+    bool mixed = false;
+    if (q < a.nq) {
         Walker w;
         Carry<NW> cw;
-        bool mixed = false;
         if (walker_init<NW>(a.P, a.in, q, w, cw)) {
             mixed = w.Lh > a.esc_lmax * w.lref;
             if (!mixed) {
@@ -255,17 +257,13 @@ __global__ void __launch_bounds__(SG_SMALL_BLOCK) k_walk_small(FwdArgs a, int mi
                 mixed = a.esc_ncross && (w.st & SG_ST_MAX_STEPS);
             }
         }
-        if (!mixed) {
-            walker_finish<NW>(a, q, w, cw);
-            return;
-        }
+        if (!mixed) walker_finish<NW>(a, q, w, cw);
     }
+    if (__ballot_sync(0xffffffffu, mixed) == 0u) return;
     a.P.max_steps = mix_max_steps;
     MixJob<NW, true> job;
     job.a = &a;
-    int st = job.start(q);
-    while (st != SG_LANE_END) st = st == SG_LANE_LIVE ? job.fast() : job.slow();
-    job.end();
+    run_lanes<MixJob<NW, true>, SG_MIX_STEPS>(job, mixed ? job.start(q) : SG_LANE_FREE);
 }
 
 #ifndef SG_MIX_MINB
@@ -768,6 +766,10 @@ int l2_bytes() {
     return cached;
 }
 
+int auto_sort(int64_t nq, int64_t nF) {
+    return nq < SG_SORT_MIN_BATCH ? 0 : (128 * nF > (int64_t)l2_bytes() / 2 ? 1 : 2);
+}
+
 sg_opts resolve(const sg_opts *o, int64_t nq, int64_t nF) {
     sg_opts r;
     sg_opts_default(&r);
@@ -779,8 +781,7 @@ sg_opts resolve(const sg_opts *o, int64_t nq, int64_t nF) {
     if (r.tau_snap <= 0.f) r.tau_snap = fminf(r.precision >= 48 ? 1e-12f : 1e-6f, r.tau_near);
     if (r.kernel == SG_KERNEL_AUTO) r.kernel = SG_KERNEL_PERSISTENT;
     if (r.sort < 0 && r.precision == 64 && r.kernel != SG_KERNEL_PLAIN && nq >= SG_SORT64_MIN_BATCH) r.sort = 2;
-    if (r.sort < 0)
-        r.sort = nq < SG_SORT_MIN_BATCH ? 0 : (128 * nF > (int64_t)l2_bytes() / 2 ? 1 : 2);
+    if (r.sort < 0) r.sort = auto_sort(nq, nF);
     if (r.kernel == SG_KERNEL_PLAIN) { r.sort = 0; r.fp64_escalate = 0; }
     return r;
 }
@@ -1138,6 +1139,11 @@ sg_status sg_exp_map(const sg_mesh *m, int64_t nq, const int32_t *mesh_id, const
     if (r.boundary_mode != 0 && r.boundary_mode != 1) return SG_ERR_INVALID_ARG;
     if (r.precision != 0 && r.precision != 32 && r.precision != 40 && r.precision != 48 && r.precision != 64)
         return SG_ERR_INVALID_ARG;
+    // (the FP64 walk's length order is a gain, not a need: a caller's workspace sized for the order that
+    // the other precisions take, or for none, is enough)
+    if ((!o || o->sort < 0) && r.precision == 64 && r.workspace &&
+        r.workspace_bytes < ws_layout(m->nF, nq, r.sort, false, r.order != nullptr).total)
+        r.sort = auto_sort(nq, m->nF);
     // The automatic precision walks in FP32 and hands long walks to the mixed walk; hole avoidance
     // has no mixed walk, so there it is the FP32 walk.
     const bool autoprec = r.precision == 0 && r.boundary_mode == 0;

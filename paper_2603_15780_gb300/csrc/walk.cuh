@@ -1261,6 +1261,29 @@ __device__ __forceinline__ void run_walks(int32_t *counter, int64_t n, Job &job)
     }
 }
 
+// The driver's tail for one task per lane (state st, FREE for a lane without one): the same hot loop and
+// service phase without tickets.  Every lane of the warp calls it.
+template <class Job, int STEPS>
+__device__ __forceinline__ void run_lanes(Job &job, int st) {
+    const unsigned FULL = 0xffffffffu;
+    bool ends = false;
+    for (;;) {
+        if (ends && st == SG_LANE_END) st = job.end();
+        if (st == SG_LANE_SLOW) st = job.slow();
+        const unsigned busy = __ballot_sync(FULL, st != SG_LANE_FREE);
+        if (busy == 0u) break;
+        unsigned live, slow;
+        do {
+#pragma unroll
+            for (int k = 0; k < STEPS; ++k)
+                if (st == SG_LANE_LIVE) st = job.fast();
+            live = __ballot_sync(FULL, st == SG_LANE_LIVE);
+            slow = __ballot_sync(FULL, st == SG_LANE_SLOW);
+        } while (live != 0u && slow == 0u);
+        ends = (live | slow) == 0u;
+    }
+}
+
 // Lanes pull task indices t < n from *counter.  A lane whose task has ended keeps its state
 // in registers until REFILL lanes of the warp are idle (each kernel sets its own threshold); then all idle lanes finish
 // (write results), take new tickets and initialise together, so the long init/finish code
