@@ -138,7 +138,8 @@ def default_opts(**kw) -> Opts:
         o = Opts()
         lib().sg_opts_default(C.byref(o))
         _defaults = bytes(o)
-    o = Opts.from_buffer_copy(_defaults)
+    o = Opts()
+    C.memmove(C.byref(o), _defaults, C.sizeof(o))
     for k, v in kw.items():
         if v is not None:
             setattr(o, k, v)
