@@ -210,8 +210,8 @@ sg_status sg_mesh_get_info(const sg_mesh *m, sg_mesh_info *info);
 /*
  * sg_mesh_update_vertices -- move the vertices of a mesh to new positions, keeping its faces
  * and adjacency, and re-derive on the device every geometric word of its walk records: the
- * per-face intrinsic shape and 3-D frame, the half-edge records, the total angle theta(x) of
- * each vertex and l_ref (Sec. 4 "Straightest geodesics": all of them are functions of the
+ * per-face intrinsic shape and 3-D frame, the half-edge records (FP32, and the FP64 geometry and
+ * double-float records of the wider walks), the total angle theta(x) of each vertex and l_ref (Sec. 4 "Straightest geodesics": all of them are functions of the
  * vertex positions; the adjacency and boundary flags depend on F only).  This serves
  * optimisation of vertex positions with the grad_V output of sg_exp_map_backward, without a
  * host round trip or a rebuild of the adjacency.
@@ -222,7 +222,9 @@ sg_status sg_mesh_get_info(const sg_mesh *m, sg_mesh_info *info);
  *           except by the first call on a mesh, which allocates O(n_vertices) FP64 scratch
  *           (cudaMalloc) that the mesh keeps until sg_mesh_destroy.
  * The records are rewritten in place: walks reading the mesh on other streams must be ordered
- * before the call by the caller.  The arithmetic is that of sg_mesh_create (FP64, no
+ * before the call by the caller, and later ones after it (one event is enough for any number of
+ * streams: a walk only reads the mesh).  The call can be captured, with or without the walks,
+ * once the first call has allocated its scratch.  The arithmetic is that of sg_mesh_create (FP64, no
  * multiply-add contraction), so an updated mesh walks like one created from the new positions;
  * the FP64 sums (theta, l_ref) are accumulated in a different order, which can move their FP32
  * values by one unit in the last place.  The faces' places on the Z-order curve that keys the
@@ -287,8 +289,7 @@ sg_status sg_exp_map(const sg_mesh *m, int64_t nq, const int32_t *mesh_id, const
  * Two more rules keep it allocation-free.  The current device must be the one the mesh was
  * created on (else SG_ERR_INVALID_ARG: the array's address is per device).  The FP64 geometry
  * and double-float records that the automatic, mixed, double-float and FP64 precisions walk on
- * are allocated by sg_mesh_create; after a vertex update they are re-derived in place, on
- * `stream`, by the next call.
+ * are allocated by sg_mesh_create and derived again, in place, by sg_mesh_update_vertices.
  */
 sg_status sg_exp_map_noalloc(const sg_mesh *m, int64_t nq, const int32_t *mesh_id, const int32_t *face,
                              const float *bary, const float *v, const float *length, int32_t n_w,

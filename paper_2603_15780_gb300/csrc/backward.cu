@@ -1186,13 +1186,7 @@ extern "C" sg_status sg_exp_map_backward(const sg_mesh *m, int32_t estimator, fl
         A.tasks = (int32_t *)(base + Lw.tasks);
         A.tasks40 = (int32_t *)(base + Lw.tasks40);
         A.rst = (int4 *)(base + Lw.rst);
-        // the wide-precision geometry of the mixed literal walks (built with the mesh; re-derived
-        // here after a vertex update)
-        sg_status st64 = sg_geom64_prepare(const_cast<sg_mesh *>(m), s, true);
-        if (st64 != SG_OK) {
-            if (own) cudaFreeAsync(ws, s);
-            return st64;
-        }
+        // the wide-precision geometry of the mixed literal walks
         P64 &Q = A.P4;
         Q.rec = m->d_rec; Q.half48 = m->d_half48; Q.half = m->d_half; Q.frm = m->d_frm; Q.rec64 = m->d_rec64;
         Q.frm64 = m->d_frm64; Q.th64 = m->d_th64; Q.fv = m->d_fv; Q.V = m->d_V; Q.face_off = m->d_face_off;

@@ -960,8 +960,9 @@ sg_status sg_mesh_create_batched(const float *V, const int64_t *v_off, const int
         return SG_ERR_OOM;
     }
     // The FP64 geometry and double-float half-edge records of the mixed, double-float and FP64
-    // walks (192 B per face, 8 B per vertex), built now so that no walk call has to allocate.
-    sg_status st64 = sg_geom64_prepare(m, 0, true);
+    // walks (192 B per face, 8 B per vertex): walk calls neither allocate nor write them.
+    sg_status st64 = sg_geom64_alloc(m);
+    if (st64 == SG_OK) st64 = sg_geom64_derive(m, nullptr);
     if (st64 == SG_OK && cudaStreamSynchronize(0) != cudaSuccess) st64 = SG_ERR_CUDA;
     if (st64 != SG_OK) {
         cudaGetLastError();
@@ -1171,15 +1172,6 @@ sg_status sg_exp_map(const sg_mesh *m, int64_t nq, const int32_t *mesh_id, const
             return st;
         }
     }
-    if (r.precision >= 40 || autoprec) {
-        // the FP64 geometry and the double-float records (built with the mesh; re-derived here
-        // after a vertex update)
-        sg_status st = sg_geom64_prepare(const_cast<sg_mesh *>(m), s, r.precision <= 48);
-        if (st != SG_OK) {
-            if (own_ws) cudaFreeAsync(own_ws, s);
-            return st;
-        }
-    }
     cudaEvent_t *pev = (cudaEvent_t *)r.prof_events;
     if (r.precision == 40) {  // the mixed walk over every query, in the chosen order
         if (pev) cudaEventRecord(pev[0], s);
@@ -1344,10 +1336,6 @@ extern "C" sg_status sg_exp_map_noalloc(const sg_mesh *m, int64_t nq, const int3
     sg_status st = sg_exp_map_workspace_size(m, nq, &r, &need);
     if (st != SG_OK) return st;
     if (need > SG_NOALLOC_SCRATCH_BYTES) return SG_ERR_OOM;
-    // The FP64 geometry and the double-float records are allocated with the mesh (a vertex update
-    // only marks them for re-derivation, which launches kernels and allocates nothing).
-    if ((r.precision == 0 || r.precision >= 40) && (!m->d_rec64 || (r.precision <= 48 && !m->d_half48)))
-        return SG_ERR_UNSUPPORTED;
     r.workspace = scratch;
     r.workspace_bytes = SG_NOALLOC_SCRATCH_BYTES;
     return sg_exp_map(m, nq, mesh_id, face, bary, v, length, n_w, w, out_face, out_bary, out_pos, out_dir, out_w,

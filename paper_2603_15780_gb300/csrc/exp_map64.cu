@@ -384,49 +384,33 @@ __global__ void k_geom64_sign(int64_t nV, const float4 *__restrict__ V, double *
 
 }  // namespace
 
-// Builds (first use) or refreshes (after a vertex update) the FP64 geometry, on `s`; with
-// half48 also the double-float half-edge records of the double-float walk.
-sg_status sg_geom64_prepare(sg_mesh *m, cudaStream_t s, bool half48) {
-    if (!m->d_rec64) {
-        const size_t b0 = sizeof(double) * 6 * (size_t)m->nF, b1 = b0, b2 = sizeof(double) * (size_t)m->nV;
-        if (cudaMalloc((void **)&m->d_rec64, b0) != cudaSuccess || cudaMalloc((void **)&m->d_frm64, b1) != cudaSuccess ||
-            cudaMalloc((void **)&m->d_th64, b2) != cudaSuccess) {
-            cudaGetLastError();
-            cudaFree(m->d_rec64); cudaFree(m->d_frm64); cudaFree(m->d_th64);
-            m->d_rec64 = m->d_frm64 = m->d_th64 = nullptr;
-            return SG_ERR_OOM;
-        }
-        m->device_bytes += (int64_t)(b0 + b1 + b2);
-        m->geom64_stale = true;
+// Device memory of the FP64 geometry and of the double-float half-edge records (mesh creation).
+sg_status sg_geom64_alloc(sg_mesh *m) {
+    const size_t b0 = sizeof(double) * 6 * (size_t)m->nF, b1 = b0, b2 = sizeof(double) * (size_t)m->nV,
+                 b3 = sizeof(int4) * 6 * (size_t)m->nF;
+    if (cudaMalloc((void **)&m->d_rec64, b0) != cudaSuccess || cudaMalloc((void **)&m->d_frm64, b1) != cudaSuccess ||
+        cudaMalloc((void **)&m->d_th64, b2) != cudaSuccess || cudaMalloc((void **)&m->d_half48, b3) != cudaSuccess) {
+        cudaGetLastError();
+        return SG_ERR_OOM;  // (the caller destroys the mesh)
     }
-    if (m->geom64_stale) {
-        if (cudaMemsetAsync(m->d_th64, 0, sizeof(double) * (size_t)m->nV, s) != cudaSuccess) return SG_ERR_CUDA;
-        k_geom64_faces<<<(unsigned)((m->nF + 255) / 256), 256, 0, s>>>(m->nF, m->d_fv, m->d_V, m->d_rec64, m->d_frm64,
-                                                                      m->d_th64);
-        k_geom64_sign<<<(unsigned)((m->nV + 255) / 256), 256, 0, s>>>(m->nV, m->d_V, m->d_th64);
-        if (cudaGetLastError() != cudaSuccess) return SG_ERR_CUDA;
-        m->geom64_stale = false;
-        m->half48_stale = true;
-    }
-    if (half48) {
-        if (!m->d_half48) {
-            const size_t b = sizeof(int4) * 6 * (size_t)m->nF;
-            if (cudaMalloc((void **)&m->d_half48, b) != cudaSuccess) {
-                cudaGetLastError();
-                m->d_half48 = nullptr;
-                return SG_ERR_OOM;
-            }
-            m->device_bytes += (int64_t)b;
-            m->half48_stale = true;
-        }
-        if (m->half48_stale) {
-            const int64_t nH = 3 * m->nF;
-            k_half48<<<(unsigned)((nH + 255) / 256), 256, 0, s>>>(nH, m->d_half, m->d_rec64, m->d_half48);
-            if (cudaGetLastError() != cudaSuccess) return SG_ERR_CUDA;
-            m->half48_stale = false;
-        }
-    }
+    m->device_bytes += (int64_t)(b0 + b1 + b2 + b3);
     return SG_OK;
+}
+
+// Derives them from the mesh's current vertices and FP32 records, on `stream`: the last part of mesh
+// creation and of every vertex update, so that a walk only ever reads them.  (Left to the first walk after
+// an update, the kernels below ran on that walk's stream: a walk on another stream, ordered after the
+// update as its caller had to, read records that were being rewritten, and a captured walk either kept
+// the records of its capture or counted as the call that had renewed them.)
+sg_status sg_geom64_derive(const sg_mesh *m, void *stream) {
+    cudaStream_t s = (cudaStream_t)stream;
+    const int64_t nH = 3 * m->nF;
+    if (cudaMemsetAsync(m->d_th64, 0, sizeof(double) * (size_t)m->nV, s) != cudaSuccess) return SG_ERR_CUDA;
+    k_geom64_faces<<<(unsigned)((m->nF + 255) / 256), 256, 0, s>>>(m->nF, m->d_fv, m->d_V, m->d_rec64, m->d_frm64,
+                                                                  m->d_th64);
+    k_geom64_sign<<<(unsigned)((m->nV + 255) / 256), 256, 0, s>>>(m->nV, m->d_V, m->d_th64);
+    k_half48<<<(unsigned)((nH + 255) / 256), 256, 0, s>>>(nH, m->d_half, m->d_rec64, m->d_half48);
+    return cudaGetLastError() == cudaSuccess ? SG_OK : SG_ERR_CUDA;
 }
 
 cudaError_t sg_launch_walk64(const sg_mesh *m, const SgFwdIO &io, int n_w, const sg_opts &r, cudaStream_t s) {

@@ -190,7 +190,6 @@ extern "C" sg_status sg_mesh_update_vertices(sg_mesh *m, const float *V, void *s
     k_update_meshes<<<(unsigned)((m->n_mesh + 127) / 128), 128, 0, s>>>(A);
     if (cudaGetLastError() != cudaSuccess) return SG_ERR_CUDA;
     m->updated = true;
-    m->geom64_stale = true;
-    m->half48_stale = true;
-    return SG_OK;
+    // the FP64 geometry and the double-float records follow on the same stream
+    return sg_geom64_derive(m, stream);
 }

@@ -68,16 +68,15 @@ struct sg_mesh {
     unsigned long long *d_ecount = nullptr;
     int *d_ndegen = nullptr;
     bool updated = false;
-    // FP64 geometry of the full-precision walk (built by its first call, refreshed after an update)
+    // FP64 geometry of the full-precision walk (allocated and derived with the mesh, derived again by
+    // every vertex update on its stream)
     double *d_rec64 = nullptr;
     double *d_frm64 = nullptr;
     double *d_th64 = nullptr;
-    bool geom64_stale = true;
     // double-float half-edge records of the double-float walk, int4[6*nF]: {l, cx} and {cy,
     // linkR, linkL} of each half-edge with every length split into two FP32 words hi + lo
-    // (built from the FP64 geometry by the walk's first call, refreshed after an update)
+    // (from the FP64 geometry, together with it)
     int4 *d_half48 = nullptr;
-    bool half48_stale = true;
 };
 
 // host-side builder (mesh_build.cpp); fills the host arrays, returns SG_OK or an error
@@ -92,6 +91,11 @@ struct sg_host_mesh {
     std::vector<double> lref64;
     std::vector<int64_t> face_off64, vert_off64;
 };
+
+// exp_map64.cu: memory of the FP64 geometry and the double-float records, and their derivation on a
+// cudaStream_t
+sg_status sg_geom64_alloc(sg_mesh *m);
+sg_status sg_geom64_derive(const sg_mesh *m, void *stream);
 
 sg_status sg_build_host_mesh(const float *V, const int64_t *v_off, const int32_t *F, const int64_t *f_off,
                              int32_t n_mesh, sg_host_mesh *out);
