@@ -412,8 +412,9 @@ sg_status sg_exp_map_steps(const sg_mesh *m, int32_t K, float h, const float *U,
  * previous step's end barycentrics.
  *   step_*     the forward's per-step records;  U, h, K, mesh_id as given to the forward
  *   g_pos      device float32 [nq][3] dL/dx_K;  g_bary  [nq][3] dL/db_K or NULL
- * Outputs (device): grad_U float32 [n_vertices][3] ACCUMULATED (+=) or NULL; grad_bary float32
- * [nq][3] dL/db_0 (meaningful up to the simplex gauge); grad_V [n_vertices][3] accumulated or NULL.
+ * Outputs (device): grad_U float32 [n_vertices][3] ACCUMULATED (+=, atomically: calls on several
+ * streams may share it) or NULL; grad_bary float32 [nq][3] dL/db_0 (meaningful up to the simplex
+ * gauge); grad_V [n_vertices][3] accumulated or NULL.
  * Scratch: sg_exp_map_steps_backward_workspace_size (o->workspace, or stream-ordered memory).
  * Asynchronous on `stream`.  Errors: as sg_exp_map_backward.
  */

@@ -237,9 +237,10 @@ __global__ void __launch_bounds__(256) k_steps_field_flush(int64_t nV, const flo
     const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (v >= nV) return;
     const float4 a = acc[v];
-    grad_U[3 * v] += a.x;
-    grad_U[3 * v + 1] += a.y;
-    grad_U[3 * v + 2] += a.z;
+    // (atomic: calls on other streams may be adding into the same array)
+    if (a.x != 0.f) atomicAdd(grad_U + 3 * v, a.x);
+    if (a.y != 0.f) atomicAdd(grad_U + 3 * v + 1, a.y);
+    if (a.z != 0.f) atomicAdd(grad_U + 3 * v + 2, a.z);
 }
 
 // The field's term of step k's VJP (see the file comment), one thread per query: gb_next[q] =
