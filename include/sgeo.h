@@ -348,10 +348,11 @@ sg_status sg_exp_map_trace(const sg_mesh *m, int64_t nq, const int32_t *mesh_id,
  *   grad_v     float32 [nq][3]  dL/dv (tangent to the start face)
  *   grad_p     float32 [nq][3]  dL/dp in the start face plane (zero for EP, Sec. 4)
  *   grad_bary  float32 [nq][3]  dL/db_k = <grad_p, x_k> (meaningful up to the simplex gauge)
- *   grad_V     float32 [nV][3]  dL/dX, ACCUMULATED (+=) over queries: the derivative of the end
- *                               point (and barycentrics) in the vertex positions with the face
- *                               sequence held fixed; queries with a vertex hit or a boundary stop
- *                               add nothing and get SG_ST_NO_GRADV
+ *   grad_V     float32 [nV][3]  dL/dX, ACCUMULATED (+=, atomically: calls on several streams may
+ *                               share it) over queries: the derivative of the end point (and
+ *                               barycentrics) in the vertex positions with the face sequence held
+ *                               fixed; queries with a vertex hit or a boundary stop add nothing and
+ *                               get SG_ST_NO_GRADV
  *   grad_w     float32 [nq][n_w][3]  dL/dw = R^T g_w (parallel transport is a rotation of the
  *                               tangent planes for a fixed face sequence; exact)
  *   out_status uint32 [nq]      SG_ST_* of the extra walks (GFD) or of the re-walk

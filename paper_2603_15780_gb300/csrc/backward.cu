@@ -1065,10 +1065,11 @@ __global__ void k_gradv_edges(int64_t nE, WalkParams P, const int2 *__restrict__
 __global__ void k_gradv_flush(int64_t nV, const float4 *__restrict__ gacc, float *grad_V) {
     int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (v >= nV) return;
-    float4 a = gacc[v];
-    grad_V[3 * v] += a.x;
-    grad_V[3 * v + 1] += a.y;
-    grad_V[3 * v + 2] += a.z;
+    const float4 a = gacc[v];
+    // (atomic: calls on other streams may be adding into the same array)
+    if (a.x != 0.f) atomicAdd(grad_V + 3 * v, a.x);
+    if (a.y != 0.f) atomicAdd(grad_V + 3 * v + 1, a.y);
+    if (a.z != 0.f) atomicAdd(grad_V + 3 * v + 2, a.z);
 }
 
 // ------------------------------------------------------------------ host

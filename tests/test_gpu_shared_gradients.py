@@ -49,3 +49,26 @@ def test_field_gradient_shared_by_streams():
                 keep.append(call(shared))
     torch.cuda.synchronize()
     _check(torch, one, shared, STREAMS * CALLS)
+
+
+@pytest.mark.parametrize("estimator", ["ep", "gfd"])
+def test_vertex_gradient_shared_by_streams(estimator):
+    torch, sg, mesh, q, cu, _ = _setup()
+    face, bary, v, g = torch.as_tensor(q.face, device="cuda"), cu(q.bary), cu(q.v), cu(q.g_pos)
+    end = sg.exp_map(mesh, face, bary, v)
+
+    def call(grad_V):
+        return sg.exp_map_backward(mesh, estimator, face, bary, v, end["face"], end["bary"], end["dir"], end["status"], g,
+                                   grad_V=grad_V)
+
+    one, shared = (torch.zeros(mesh.n_vertices, 3, device="cuda") for _ in range(2))
+    call(one)
+    torch.cuda.synchronize()
+    assert float(one.abs().max()) > 0
+    streams, keep = [torch.cuda.Stream() for _ in range(STREAMS)], []
+    for i in range(CALLS):
+        for s in streams:
+            with torch.cuda.stream(s):
+                keep.append(call(shared))
+    torch.cuda.synchronize()
+    _check(torch, one, shared, STREAMS * CALLS)
