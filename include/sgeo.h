@@ -278,8 +278,9 @@ sg_status sg_exp_map(const sg_mesh *m, int64_t nq, const int32_t *mesh_id, const
  * Same arguments, outputs and errors as sg_exp_map; o->workspace is ignored.  The scratch
  * (work-queue counter and start-face sort) lives in one fixed 32 MiB device array inside the
  * library, which every GPU that loads the library holds until the process exits.  Batches
- * whose scratch (sg_exp_map_workspace_size with the same options) exceeds 32 MiB are rejected
- * with SG_ERR_OOM and nothing is launched; with o->sort = 0 the scratch is 64 bytes and any
+ * whose scratch (sg_exp_map_workspace_size with the same options; for precision 64 and an
+ * automatic order the smaller of its length order and the other precisions' order) exceeds 32 MiB
+ * are rejected with SG_ERR_OOM and nothing is launched; with o->sort = 0 the scratch is 64 bytes and any
  * batch size fits.  No cudaMalloc, cudaFree or allocating library routine is called.
  * The first call on a device looks the array's address up (cudaGetSymbolAddress) with that
  * device current; make that first call before any stream capture.  All calls share the one

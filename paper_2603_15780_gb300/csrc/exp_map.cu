@@ -770,6 +770,10 @@ int auto_sort(int64_t nq, int64_t nF) {
     return nq < SG_SORT_MIN_BATCH ? 0 : (128 * nF > (int64_t)l2_bytes() / 2 ? 1 : 2);
 }
 
+// The FP64 walk's length order is a gain, not a need: scratch sized for the order that the other precisions
+// take (auto_sort), or for none, is enough, whether a caller's workspace or the allocation-free array.
+bool wants_sort64(const sg_opts &o) { return o.sort < 0 && o.precision == 64 && o.kernel != SG_KERNEL_PLAIN; }
+
 sg_opts resolve(const sg_opts *o, int64_t nq, int64_t nF) {
     sg_opts r;
     sg_opts_default(&r);
@@ -780,7 +784,7 @@ sg_opts resolve(const sg_opts *o, int64_t nq, int64_t nF) {
     if (r.tau_near <= 0.f) r.tau_near = 1e-4f;
     if (r.tau_snap <= 0.f) r.tau_snap = fminf(r.precision >= 48 ? 1e-12f : 1e-6f, r.tau_near);
     if (r.kernel == SG_KERNEL_AUTO) r.kernel = SG_KERNEL_PERSISTENT;
-    if (r.sort < 0 && r.precision == 64 && r.kernel != SG_KERNEL_PLAIN && nq >= SG_SORT64_MIN_BATCH) r.sort = 2;
+    if (wants_sort64(r) && nq >= SG_SORT64_MIN_BATCH) r.sort = 2;
     if (r.sort < 0) r.sort = auto_sort(nq, nF);
     if (r.kernel == SG_KERNEL_PLAIN) { r.sort = 0; r.fp64_escalate = 0; }
     return r;
@@ -1140,10 +1144,8 @@ sg_status sg_exp_map(const sg_mesh *m, int64_t nq, const int32_t *mesh_id, const
     if (r.boundary_mode != 0 && r.boundary_mode != 1) return SG_ERR_INVALID_ARG;
     if (r.precision != 0 && r.precision != 32 && r.precision != 40 && r.precision != 48 && r.precision != 64)
         return SG_ERR_INVALID_ARG;
-    // (the FP64 walk's length order is a gain, not a need: a caller's workspace sized for the order that
-    // the other precisions take, or for none, is enough)
-    if ((!o || o->sort < 0) && r.precision == 64 && r.workspace &&
-        r.workspace_bytes < ws_layout(m->nF, nq, r.sort, false, r.order != nullptr).total)
+    if (o && o->workspace && wants_sort64(*o) &&
+        o->workspace_bytes < ws_layout(m->nF, nq, r.sort, false, r.order != nullptr).total)
         r.sort = auto_sort(nq, m->nF);
     // The automatic precision walks in FP32 and hands long walks to the mixed walk; hole avoidance
     // has no mixed walk, so there it is the FP32 walk.
@@ -1334,6 +1336,10 @@ extern "C" sg_status sg_exp_map_noalloc(const sg_mesh *m, int64_t nq, const int3
     if (o) r = *o;
     size_t need = 0;
     sg_status st = sg_exp_map_workspace_size(m, nq, &r, &need);
+    if (st == SG_OK && need > SG_NOALLOC_SCRATCH_BYTES && wants_sort64(r)) {
+        r.sort = auto_sort(nq, m->nF);
+        st = sg_exp_map_workspace_size(m, nq, &r, &need);
+    }
     if (st != SG_OK) return st;
     if (need > SG_NOALLOC_SCRATCH_BYTES) return SG_ERR_OOM;
     r.workspace = scratch;

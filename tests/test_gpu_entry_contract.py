@@ -1,0 +1,57 @@
+"""What the entry points accept and how they launch: scratch limits, launch options."""
+import ctypes as C
+
+import numpy as np
+import pytest
+
+import meshgen
+
+pytestmark = pytest.mark.gpu
+
+OUT = (("face", "int32", ()), ("bary", "float32", (3,)), ("pos", "float32", (3,)), ("dir", "float32", (3,)),
+       ("status", "int32", ()), ("ncross", "int32", ()), ("hash", "int64", ()))
+
+
+def _outputs(n):
+    import torch
+    return {k: torch.zeros((n, *s), dtype=getattr(torch, d), device="cuda") for k, d, s in OUT}
+
+
+def _call(fn, mesh, face, bary, v, opts, out, stream=None):
+    """sg_exp_map or sg_exp_map_noalloc into `out`; the status."""
+    p = lambda k: out[k].data_ptr()
+    return fn(mesh.handle, face.numel(), None, face.data_ptr(), bary.data_ptr(), v.data_ptr(), None, 0, None, p("face"),
+              p("bary"), p("pos"), p("dir"), None, p("status"), p("ncross"), p("hash"), C.byref(opts), stream)
+
+
+def _inputs(X, F, n, lo, hi, seed=5):
+    import torch
+
+    import paper_2603_15780_gb300 as sg
+    rng = np.random.Generator(np.random.PCG64(seed))
+    q = meshgen.sample_queries(X, F, n, rng, lo, hi, 0)
+    cu = lambda x: torch.as_tensor(np.ascontiguousarray(x, np.float32), device="cuda")
+    return sg, sg.Mesh(X.astype(np.float32), F), (torch.as_tensor(q.face, device="cuda"), cu(q.bary), cu(q.v))
+
+
+@pytest.mark.parametrize("n,fits", [(7_200_000, True), (7_900_000, False)])
+def test_noalloc_takes_fp64_batches_of_the_start_face_order(n, fits):
+    """On 600,000 faces the 32 MiB hold the length order (5 bytes a query) of 6.7M queries and the
+    start-face order (4 bytes a query and a face) of 7.8M: between the two the FP64 walk falls back to the
+    second."""
+    import torch
+    X, F = meshgen.torus(600, 500)
+    sg, mesh, few = _inputs(X, F, 4000, 0.0, 0.01)
+    face, bary, v = (x.repeat(n // 4000, *[1] * (x.dim() - 1)).contiguous() for x in few)
+    out = _outputs(n)
+    rc = _call(sg.lib().sg_exp_map_noalloc, mesh, face, bary, v, sg.default_opts(precision=64), out)
+    assert rc == (0 if fits else 5)                                   # 5: SG_ERR_OOM
+    torch.cuda.synchronize()
+    if not fits:
+        assert not bool(out["hash"].any())                            # nothing was launched
+        return
+    ref = sg.exp_map(mesh, *few, precision=64, want_hash=True)
+    torch.cuda.synchronize()
+    for k, _, s in OUT:
+        a = out[k].reshape(n // 4000, 4000, *s)
+        assert torch.equal(a, ref[k].reshape(1, 4000, *s).expand_as(a)), k
