@@ -97,7 +97,8 @@ typedef struct sg_opts {
                                always in input order.  sg_exp_map_backward's re-walk uses the
                                length order when sort is 2, or auto with >= 65536 queries. */
     int32_t block;          /* threads per block; <= 0: 256 */
-    int32_t blocks_per_sm;  /* persistent kernel residency; <= 0: as many as fit */
+    int32_t blocks_per_sm;  /* persistent kernel residency; <= 0: as many as fit.  Precision 48 and 64
+                               count blocks of 128 threads */
     int32_t fp64_escalate;  /* 1: re-evaluate near-vertex classification in FP64 (persistent only) */
     float tau_near;         /* flag radius / l_ref for NEAR_VERTEX, NEAR_EDGE and the FP64 band; <= 0: 1e-4 */
     float tau_snap;         /* vertex-snap radius / l_ref; <= 0: 1e-6 (precision 0, 32, 40), 1e-12

@@ -428,8 +428,13 @@ cudaError_t sg_launch_walk64(const sg_mesh *m, const SgFwdIO &io, int n_w, const
     const int sms = sg_sm_count();
     auto go = [&](auto kern, auto per_sm) {
         // A batch that leaves SMs idle in blocks of 128 takes blocks of one warp, dealt evenly over the
-        // SMs with the longest walks first: the FP64 units, one per SM partition, bound the walk
-        const int block = io.nq < (int64_t)sms * 128 * 4 ? 32 : 128;
+        // SMs with the longest walks first: the FP64 units, one per SM partition, bound the walk.  The line
+        // is four blocks of 128 per SM (FP64 / double-float walk, blocks of 128 and of 32 threads, 500 to
+        // 64,000 queries on a 65,536-face torus: 327 -> 315 / 154 -> 138 us at 500, 388 -> 376 / 165 -> 158
+        // at 8,000, 643 -> 604 / 204 -> 199 at 40,000, 911 -> 903 / 262 -> 256 at 64,000).  A caller's
+        // blocks_per_sm counts blocks of 128 (one block of a warp per SM instead: 1.07 and 2.4 times the time
+        // at 64,000).
+        const int block = r.blocks_per_sm <= 0 && io.nq < (int64_t)sms * 128 * 4 ? 32 : 128;
         const int per = r.blocks_per_sm > 0 ? r.blocks_per_sm : per_sm(block);
         const int64_t grid = std::min<int64_t>((int64_t)sms * per, std::max<int64_t>((io.nq + block - 1) / block, 1));
         kern<<<(unsigned)grid, block, 0, s>>>(a);

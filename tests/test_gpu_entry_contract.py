@@ -34,6 +34,37 @@ def _inputs(X, F, n, lo, hi, seed=5):
     return sg, sg.Mesh(X.astype(np.float32), F), (torch.as_tensor(q.face, device="cuda"), cu(q.bary), cu(q.v))
 
 
+def _kernels(launch):
+    """(grid, block) of each kernel that `launch(stream)` enqueues, from a stream capture (nothing runs)."""
+    import torch
+
+    class Params(C.Structure):
+        _fields_ = [("func", C.c_void_p), ("grid", C.c_uint * 3), ("block", C.c_uint * 3), ("shared", C.c_uint),
+                    ("params", C.c_void_p), ("extra", C.c_void_p), ("kern", C.c_void_p), ("ctx", C.c_void_p)]
+    cu = C.CDLL("libcuda.so.1")
+    s = torch.cuda.Stream()
+    stream, graph, n, kind = C.c_void_p(s.cuda_stream), C.c_void_p(), C.c_size_t(), C.c_int()
+    torch.cuda.synchronize()
+    assert cu.cuStreamBeginCapture_v2(stream, C.c_int(2)) == 0       # (relaxed)
+    try:
+        rc = launch(s.cuda_stream)
+    finally:
+        end = cu.cuStreamEndCapture(stream, C.byref(graph))
+    assert rc == 0 and end == 0
+    assert cu.cuGraphGetNodes(graph, None, C.byref(n)) == 0
+    nodes = (C.c_void_p * n.value)()
+    assert cu.cuGraphGetNodes(graph, nodes, C.byref(n)) == 0
+    out = []
+    for x in nodes:
+        assert cu.cuGraphNodeGetType(C.c_void_p(x), C.byref(kind)) == 0
+        if kind.value == 0:
+            k = Params()
+            assert cu.cuGraphKernelNodeGetParams_v2(C.c_void_p(x), C.byref(k)) == 0
+            out.append((k.grid[0], k.block[0]))
+    cu.cuGraphDestroy(graph)
+    return out
+
+
 @pytest.mark.parametrize("n,fits", [(7_200_000, True), (7_900_000, False)])
 def test_noalloc_takes_fp64_batches_of_the_start_face_order(n, fits):
     """On 600,000 faces the 32 MiB hold the length order (5 bytes a query) of 6.7M queries and the
@@ -55,3 +86,17 @@ def test_noalloc_takes_fp64_batches_of_the_start_face_order(n, fits):
     for k, _, s in OUT:
         a = out[k].reshape(n // 4000, 4000, *s)
         assert torch.equal(a, ref[k].reshape(1, 4000, *s).expand_as(a)), k
+
+
+@pytest.mark.parametrize("precision", [48, 64])
+def test_wide_walk_keeps_the_residency_it_is_given(precision):
+    """blocks_per_sm counts blocks of 128 threads at every batch size."""
+    import torch
+    X, F = meshgen.icosphere(2)
+    sg, mesh, q = _inputs(X, F, 20000, 0.0, 0.1)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    out, ws = _outputs(20000), torch.empty(4096, dtype=torch.uint8, device="cuda")
+    for per in (1, 2):
+        opts = sg.default_opts(precision=precision, sort=0, blocks_per_sm=per, workspace=ws.data_ptr(), workspace_bytes=4096)
+        got = _kernels(lambda s: _call(sg.lib().sg_exp_map, mesh, *q, opts, out, s))
+        assert got == [(min(sms * per, -(-20000 // 128)), 128)]
