@@ -96,7 +96,9 @@ typedef struct sg_opts {
                                than 768 l_ref come first, longest first.  Outputs are
                                always in input order.  sg_exp_map_backward's re-walk uses the
                                length order when sort is 2, or auto with >= 65536 queries. */
-    int32_t block;          /* threads per block; <= 0: 256 */
+    int32_t block;          /* threads per block of the forward walk, a multiple of 32 up to 256; <= 0:
+                               256.  In a small batch on the AUTO kernel 256 leaves the choice to the
+                               library (128); precision 40, 48 and 64 use blocks of their own */
     int32_t blocks_per_sm;  /* persistent kernel residency; <= 0: as many as fit.  Precision 48 and 64
                                count blocks of 128 threads */
     int32_t fp64_escalate;  /* 1: re-evaluate near-vertex classification in FP64 (persistent only) */

@@ -48,7 +48,8 @@
 #ifndef SG_MIX_REFILL
 #define SG_MIX_REFILL 8
 #endif
-// threads per block of a small batch's walk (20k queries: 32 24.8, 64 24.8, 128 24.3, 256 25.5 us)
+// threads per block of a small batch's walk when the caller leaves the choice to the library (20k queries:
+// 32 24.8, 64 24.8, 128 24.3, 256 25.5 us)
 #ifndef SG_SMALL_BLOCK
 #define SG_SMALL_BLOCK 128
 #endif
@@ -1165,7 +1166,10 @@ sg_status sg_exp_map(const sg_mesh *m, int64_t nq, const int32_t *mesh_id, const
     a.out_w = out_w; a.out_status = out_status; a.out_ncross = out_ncross; a.out_hash = out_hash;
 
     const bool persistent = r.kernel == SG_KERNEL_PERSISTENT;
-    const bool small = auto_kernel && autoprec && !persistent && r.fp64_escalate && r.queries_per_thread <= 1;
+    // (256 threads, the default options' value, are not a choice of the caller's; other blocks above
+    // SG_SMALL_BLOCK, which k_walk_small is not compiled for, are launched as they were given)
+    const bool small = auto_kernel && autoprec && !persistent && r.fp64_escalate && r.queries_per_thread <= 1 &&
+                       (r.block <= SG_SMALL_BLOCK || r.block == 256);
     void *own_ws = nullptr;
     if (persistent || (autoprec && !small) || r.order) {
         sg_status st = prepare_queue(m, nq, mesh_id, face, r, persistent ? r.sort : 0, s, a, &own_ws, autoprec);
@@ -1201,13 +1205,14 @@ sg_status sg_exp_map(const sg_mesh *m, int64_t nq, const int32_t *mesh_id, const
     if (pev) cudaEventRecord(pev[0], s);
     cudaError_t e;
     if (small) {
-        const unsigned grid = (unsigned)((nq + SG_SMALL_BLOCK - 1) / SG_SMALL_BLOCK);
+        const int block = std::min(r.block, SG_SMALL_BLOCK);
+        const unsigned grid = (unsigned)((nq + block - 1) / block);
         switch (n_w) {
-            case 0: k_walk_small<0><<<grid, SG_SMALL_BLOCK, 0, s>>>(a, r.max_steps); break;
-            case 1: k_walk_small<1><<<grid, SG_SMALL_BLOCK, 0, s>>>(a, r.max_steps); break;
-            case 2: k_walk_small<2><<<grid, SG_SMALL_BLOCK, 0, s>>>(a, r.max_steps); break;
-            case 3: k_walk_small<3><<<grid, SG_SMALL_BLOCK, 0, s>>>(a, r.max_steps); break;
-            default: k_walk_small<4><<<grid, SG_SMALL_BLOCK, 0, s>>>(a, r.max_steps); break;
+            case 0: k_walk_small<0><<<grid, block, 0, s>>>(a, r.max_steps); break;
+            case 1: k_walk_small<1><<<grid, block, 0, s>>>(a, r.max_steps); break;
+            case 2: k_walk_small<2><<<grid, block, 0, s>>>(a, r.max_steps); break;
+            case 3: k_walk_small<3><<<grid, block, 0, s>>>(a, r.max_steps); break;
+            default: k_walk_small<4><<<grid, block, 0, s>>>(a, r.max_steps); break;
         }
         e = cudaGetLastError();
     } else switch (n_w) {

@@ -100,3 +100,20 @@ def test_wide_walk_keeps_the_residency_it_is_given(precision):
         opts = sg.default_opts(precision=precision, sort=0, blocks_per_sm=per, workspace=ws.data_ptr(), workspace_bytes=4096)
         got = _kernels(lambda s: _call(sg.lib().sg_exp_map, mesh, *q, opts, out, s))
         assert got == [(min(sms * per, -(-20000 // 128)), 128)]
+
+
+@pytest.mark.parametrize("block,want", [(32, 32), (64, 64), (128, 128), (192, 192), (256, 128), (0, 128)])
+def test_small_batch_launches_the_block_it_is_given(block, want):
+    """(256 is the default options' value: the library's own choice.  Above 128 threads the walk that goes
+    on in the mixed arithmetic is a second launch.)"""
+    import torch
+    X, F = meshgen.icosphere(2)
+    sg, mesh, q = _inputs(X, F, 1000, 0.0, 1.0)
+    ref = sg.exp_map(mesh, *q, want_hash=True)
+    opts = sg.default_opts(block=block)
+    out = _outputs(1000)
+    got = _kernels(lambda s: _call(sg.lib().sg_exp_map, mesh, *q, opts, out, s))
+    assert got[0] == (-(-1000 // want), want) and len(got) == (2 if want > 128 else 1)
+    rc = _call(sg.lib().sg_exp_map, mesh, *q, opts, out)
+    torch.cuda.synchronize()
+    assert rc == 0 and all(torch.equal(out[k], ref[k]) for k, _, _ in OUT)
