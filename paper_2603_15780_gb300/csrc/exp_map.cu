@@ -1170,6 +1170,10 @@ sg_status sg_exp_map(const sg_mesh *m, int64_t nq, const int32_t *mesh_id, const
     // SG_SMALL_BLOCK, which k_walk_small is not compiled for, are launched as they were given)
     const bool small = auto_kernel && autoprec && !persistent && r.fp64_escalate && r.queries_per_thread <= 1 &&
                        (r.block <= SG_SMALL_BLOCK || r.block == 256);
+    // (the one launch of a small batch needs no scratch, but a workspace that is given has the size that
+    // sg_exp_map_workspace_size states, whichever way the call takes)
+    if (small && r.workspace && r.workspace_bytes < ws_layout(m->nF, nq, 0, true, r.order != nullptr).total)
+        return SG_ERR_OOM;
     void *own_ws = nullptr;
     if (persistent || (autoprec && !small) || r.order) {
         sg_status st = prepare_queue(m, nq, mesh_id, face, r, persistent ? r.sort : 0, s, a, &own_ws, autoprec);

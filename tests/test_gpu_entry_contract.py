@@ -117,3 +117,16 @@ def test_small_batch_launches_the_block_it_is_given(block, want):
     rc = _call(sg.lib().sg_exp_map, mesh, *q, opts, out)
     torch.cuda.synchronize()
     assert rc == 0 and all(torch.equal(out[k], ref[k]) for k, _, _ in OUT)
+
+
+def test_small_batch_refuses_a_workspace_that_is_too_small():
+    import torch
+    X, F = meshgen.icosphere(2)
+    sg, mesh, q = _inputs(X, F, 1000, 0.0, 1.0)
+    need = sg.workspace_size(mesh, 1000, sg.default_opts())
+    ws = torch.empty(need, dtype=torch.uint8, device="cuda")
+    for size, want in ((need, 0), (need - 1, 5), (64, 5)):
+        out = _outputs(1000)
+        rc = _call(sg.lib().sg_exp_map, mesh, *q, sg.default_opts(workspace=ws.data_ptr(), workspace_bytes=size), out)
+        torch.cuda.synchronize()
+        assert rc == want and bool(out["hash"].any()) == (want == 0)
