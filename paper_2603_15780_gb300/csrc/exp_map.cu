@@ -498,9 +498,12 @@ __device__ __forceinline__ float query_length(const QueryIn &in, int64_t i) {
 
 // Key of query i: the spatial rank of its start face (its place on its mesh's Z-order curve of
 // face centroids, offset by the mesh's first face); nF for an invalid query.  With the automatic
-// precision (esc_lmax > 0) the queries longer than esc_lmax l_ref, which the mixed walk takes,
-// keep that rank as key and form the permutation's head; the others get nF + the rank, and an
-// invalid query 2 nF.  On meshes of SG_FAR_MIN_FACES and more, the head's head are the walks longer than
+// precision (esc_lmax > 0) the queries longer than esc_lmax l_ref, which the mixed walk takes, form the
+// permutation's head: face_head_keys() keys, below SG_FAR_MIN_FACES that rank; the others get that many plus
+// the rank, and an invalid query that many plus nF.  The histogram and the scatter both evaluate the key
+// and have to agree to the last bit: no product meets a sum here or in query_length but in an explicit
+// fmaf, so nothing is left to the compiler's contraction.
+// On meshes of SG_FAR_MIN_FACES and more, the head's head are the walks longer than
 // SG_FAR_LREF l_ref, by length (a quarter of an octave per class, longest first), then place (1024 cells):
 // thousands of crossings leave the neighbourhood of the start at once, so starting together gains them
 // little, and one that starts late ends alone.  To make room for their keys the head's other queries
@@ -1077,8 +1080,7 @@ sg_status prepare_queue(const sg_mesh *m, int64_t nq, const int32_t *mesh_id, co
         a.esc_list = (int32_t *)(base + L.esc);
         a.esc_count = a.counter + SG_CTR_ESC;
     }
-    // with the automatic precision the orders route the long queries to the mixed walk (the
-    // length order's head, the start-face order's tail)
+    // with the automatic precision the orders route the long queries, their head, to the mixed walk
     const float lmax = esc ? SG_AUTO_FP32_LREF : 0.f;
     // A caller's order buffer (sg_opts.order) receives the length order: the queue's own when it
     // takes the queries in that order, else one built for the buffer after the queue's

@@ -31,28 +31,20 @@ struct FaceRec {
     float l01, x2x, x2y, il1, il2;
 };
 
-// One 32-byte record = one L2 sector, read with one 256-bit load (sm_100 and later) or, without W, as
-// two 16-byte loads.  The wide load halves the requests per record and doubles the device's
-// dependent-gather ceiling: the half-edge record of every crossing (1M queries on an 81,920-face
+// One 32-byte record = one L2 sector, read with one 256-bit load (sm_100 and later).  Against two 16-byte
+// loads it halves the requests per record and doubles the device's dependent-gather ceiling: the half-edge record of every crossing (1M queries on an 81,920-face
 // sphere, queries in walk-length order: forward walk 0.437 -> 0.404 ms, backward re-walk 0.738 -> 0.716
 // ms, whose L2 tag lookups had run at 74% with two 16-byte loads and an atomic per crossing), and the
 // face records and frames that the elementwise kernels gather (k_bwd_assemble 64 -> 57 us on 1M queries).
-template <bool W = true>
 __device__ __forceinline__ void ld_rec32(const int4 *__restrict__ p, int4 &a, int4 &b) {
-    if (W) {
-        asm("ld.global.nc.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-            : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
-            : "l"(p));
-    } else {
-        a = __ldg(p);
-        b = __ldg(p + 1);
-    }
+    asm("ld.global.nc.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+        : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
+        : "l"(p));
 }
 
-template <bool W = true>
 __device__ __forceinline__ FaceRec load_rec(const int4 *__restrict__ rec, int f) {
     int4 a, b;
-    ld_rec32<W>(rec + 2 * f, a, b);
+    ld_rec32(rec + 2 * f, a, b);
     FaceRec r;
     r.n0 = a.x; r.n1 = a.y; r.n2 = a.z;
     r.l01 = __int_as_float(a.w);
@@ -717,7 +709,7 @@ __device__ __forceinline__ bool half_step(Walker &w, const WalkParams &P, Hook &
         ndx = (fl ? da : -da) * re; ndy = dc * re;
         eda = da; edc = dc;
     }
-    const FaceRec G = load_rec<true>(MIX ? P.half48 : P.half, hn);
+    const FaceRec G = load_rec(MIX ? P.half48 : P.half, hn);
     if (!MIX) {
         const int k = w.h - 3 * (w.h / 3);
         const int g = hn / 3;
@@ -772,7 +764,7 @@ __device__ __forceinline__ int fast_step(Walker &w, const WalkParams &P, Hook &h
     hook.on_apex(w, sC, cx, cy, x, 0.f);
     if (end) return SG_FAST_END;
     const int hn = link >> 1, fl = link & 1;
-    const FaceRec G = load_rec<true>(MIX ? P.half48 : P.half, hn);
+    const FaceRec G = load_rec(MIX ? P.half48 : P.half, hn);
     {   // compensated L -= t (see half_step)
         const float sum = w.Lh - t;
         w.Ll += -t - (sum - w.Lh);
@@ -833,12 +825,13 @@ __device__ __forceinline__ bool walker_step(Walker &w, const WalkParams &P, Hook
     return general_step<ESC, HOLE, MIX>(w, P, hook);
 }
 
-// One step of a walk kernel.  Returns true when the walk is finished, except for half_final, which
+// One step of a kernel that walks one query per thread.  Returns true when the walk is finished, except for half_final, which
 // the caller owes a walk that ended in the half-edge mode (walker_settle, before its end is read).
-template <bool ESC, bool HOLE = false, bool MIX = false, class Hook = NoHook>
-__device__ __forceinline__ bool walker_advance(Walker &w, const WalkParams &P, Hook &&hook = Hook()) {
-    const int r = fast_step<MIX, true>(w, P, hook);
-    return r == SG_FAST_SLOW ? walker_step<ESC, HOLE, MIX>(w, P, hook) : r == SG_FAST_END;
+template <bool ESC>
+__device__ __forceinline__ bool walker_advance(Walker &w, const WalkParams &P) {
+    NoHook hook;
+    const int r = fast_step<false, true>(w, P, hook);
+    return r == SG_FAST_SLOW ? walker_step<ESC>(w, P) : r == SG_FAST_END;
 }
 // the lane state of a walk that is about to take a step: an ordinary crossing is possible from the
 // half-edge mode only
@@ -956,7 +949,7 @@ __device__ __forceinline__ bool general_step(Walker &w, const WalkParams &P, Hoo
     const float da = fmaf(w.dx, ex, w.dy * ey);
     const float dc = fmaf(w.dx, ey, -w.dy * ex);  // d . (ey, -ex)
     const int hn = 3 * g + kp;
-    const FaceRec G = load_rec<true>(MIX ? P.half48 : P.half, hn);
+    const FaceRec G = load_rec(MIX ? P.half48 : P.half, hn);
     float ndx = fl ? da : -da, ndy = dc;
     renorm(ndx, ndy);
     if (MIX) {  // a face-frame step (a start on an edge or vertex, a vertex transport) is FP32
@@ -1137,7 +1130,7 @@ __device__ __forceinline__ void walker_start_mix(const WalkParams &P, const Quer
     const float b0 = __ldg(in.bary + 3 * q), b1 = __ldg(in.bary + 3 * q + 1), b2 = __ldg(in.bary + 3 * q + 2);
     if (!(b0 > 0.f && b1 > 0.f && b2 > 0.f)) return;
     int4 ra, rb;
-    ld_rec32<true>(P.half48 + 2 * (3 * w.f), ra, rb);  // half-edge 0 of the face: its frame is the face's
+    ld_rec32(P.half48 + 2 * (3 * w.f), ra, rb);  // half-edge 0 of the face: its frame is the face's
     const DF l01{__int_as_float(ra.x), __int_as_float(ra.y)}, x2x{__int_as_float(ra.z), __int_as_float(ra.w)};
     const DF x2y{__int_as_float(rb.x), __int_as_float(rb.y)};
     const DF sb = df_add(two_sum(b0, b1), DF{b2, 0.f});
@@ -1185,7 +1178,7 @@ __device__ __forceinline__ void walker_start_mix(const WalkParams &P, const Quer
     if (!(hy.hi > 0.f)) return;
     const DF Lx = df_add_same_sign(L, tb);
     w.h = 3 * w.f + j;
-    w.R = load_rec<true>(P.half48, w.h);
+    w.R = load_rec(P.half48, w.h);
     w.px = se.hi; w.py = 0.f;
     w.dx = hx.hi; w.dxl = hx.lo;
     w.dy = hy.hi; w.dyl = hy.lo;
@@ -1222,8 +1215,15 @@ __device__ __forceinline__ int64_t fetch_ticket(int32_t *counter) {
 // at the start, a rare step is served at once, and ended walks wait until no lane of the warp walks:
 // they have no successor to make room for, and serving them one by one, each a chain of dependent
 // loads, held up the lanes still walking (20k queries: re-walk 47 -> 38 us, literal walks 41 -> 34 us; trace of
-// 10k 49 -> 34 us).  The control is uniform over the warp and every vote is taken by all of its lanes
-// in straight line, none behind a condition.
+// 10k 49 -> 34 us).
+// Why it ends: `exhausted`, `live`, `slow` and `busy` come from ballots and are the same on every lane; each
+// turn of the outer loop ends, serves or starts at least one walk, or takes a ticket past n; and each walk
+// is bounded by its step cap.  Why the votes stand where they do: a full-mask vote is defined only when
+// all 32 lanes reach that same vote.  An earlier form of the tail rule took votes behind short-circuit
+// conditions (`!exhausted || !__any_sync(...)`), whose operands are equal on all lanes but which the
+// compiler need not know to be, and it may then let lanes reach them by different paths; that form hung
+// once, in the backward, for a reason that was not established beyond this.  So every vote is
+// unconditional, in straight line, kept in a ballot word, and conditions are formed from the words.
 // Job: int init(t), end(), slow(), each returning the lane's new state (init and end write the
 // outputs of a task that is done); int fast() returns SG_FAST_*.  STEPS crossings run
 // between looks at the lanes' states.
@@ -1283,21 +1283,15 @@ __device__ __forceinline__ void run_lanes(Job &job, int st) {
     }
 }
 
-// Lanes pull task indices t < n from *counter.  A lane whose task has ended keeps its state
-// in registers until REFILL lanes of the warp are idle (each kernel sets its own threshold); then all idle lanes finish
+// The hole-avoidance walk's driver.  Lanes pull task indices t < n from *counter.  A lane whose task has
+// ended keeps its state in registers until REFILL lanes of the warp are idle; then all idle lanes finish
 // (write results), take new tickets and initialise together, so the long init/finish code
 // runs with many lanes active instead of stalling the warp for one lane every few steps.
 // Once the counter passes n, lanes finish as soon as they are done and the warp leaves when
 // all of its lanes are idle.  Every lane of the warp stays in the loop until then (the
 // ballots use the full mask).  Job: bool init(t) (true: a walk to step), bool step()
-// (true: done), void finish().  STEPS walk steps run between refill checks (each kernel sets
-// its own count).
-#define SG_REFILL_LANES 8
-#ifndef SG_STEPS_PER_CHECK
-#define SG_STEPS_PER_CHECK 2
-#endif
-
-template <class Job, int REFILL = SG_REFILL_LANES, int STEPS = SG_STEPS_PER_CHECK>
+// (true: done), void finish().  STEPS walk steps run between refill checks.
+template <class Job, int REFILL, int STEPS>
 __device__ __forceinline__ void run_persistent(int32_t *counter, int64_t n, Job &job) {
     if (n <= 0) return;  // an empty list (a count read from device memory): no ticket to take
     bool live = false, pending = false, exhausted = false;

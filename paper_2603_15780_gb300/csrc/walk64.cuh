@@ -67,9 +67,6 @@ __device__ __forceinline__ void hash64(W64 &w, int f, int want) {
         w.hash *= SG_FNV_PRIME;
     }
 }
-__device__ __forceinline__ double sig64(const W64 &w, double cx, double cy) {
-    return w.dx * (cy - w.py) - w.dy * (cx - w.px);
-}
 __device__ __forceinline__ void norm2(double &x, double &y) {
     const double r = 1.0 / sqrt(x * x + y * y);
     x *= r; y *= r;
@@ -266,7 +263,7 @@ __device__ bool step64(W64 &w, const P64 &P) {
 // the double-float half-edge record h into R: one 32-byte sector, one 256-bit load
 __device__ __forceinline__ void load48(R64 &R, const P64 &P, int h) {
     int4 a, b;
-    ld_rec32<true>(P.half48 + 2 * h, a, b);
+    ld_rec32(P.half48 + 2 * h, a, b);
     R.l01 = dpack(DF{__int_as_float(a.x), __int_as_float(a.y)});
     R.x2x = dpack(DF{__int_as_float(a.z), __int_as_float(a.w)});
     R.x2y = dpack(DF{__int_as_float(b.x), __int_as_float(b.y)});
