@@ -54,7 +54,7 @@
 #define SG_SMALL_BLOCK 128
 #endif
 // the hole-avoidance walk keeps the older driver (run_persistent), whose boundary events wait for
-// each other (SG_HOLE_BATCH): on run_walks it took 0.98-1.11 ms against 0.72 ms on 262k queries
+// each other (SG_HOLE_BATCH): on run_walks it took 0.79-1.06 ms against 0.52 ms on 262k queries
 #ifndef SG_HOLE_REFILL
 #define SG_HOLE_REFILL 12
 #endif
@@ -507,9 +507,12 @@ __device__ __forceinline__ float query_length(const QueryIn &in, int64_t i) {
 // SG_FAR_LREF l_ref, by length (a quarter of an octave per class, longest first), then place (1024 cells):
 // thousands of crossings leave the neighbourhood of the start at once, so starting together gains them
 // little, and one that starts late ends alone.  To make room for their keys the head's other queries
-// share a key in pairs of ranks.  (A 2.1M-face heightfield, 524k queries, the whole call: lengths up to 3,300
-// l_ref 9.16 -> 7.99 ms, up to 1,650 6.38 -> 5.79, up to 1,100 5.17 -> 4.94.  The line: up to 660 l_ref
-// 3.61 ms by place, 3.66 by length first; up to 330, 3.28 against 3.80; up to 55, 0.67 against 0.92.)
+// share a key in pairs of ranks.  (524k queries with lengths uniform up to the stated bound, the whole call,
+// without and with these classes.  Up to 3,300 l_ref: heightfield of 2.1M faces 9.57 -> 8.59 ms, torus of 2.1M
+// 24.97 -> 22.02, sphere of 1.3M 18.81 -> 16.41; up to 1,650: 7.02 -> 6.38, 12.51 -> 11.84, 9.48 -> 8.78; up
+// to 1,100: 5.59 -> 5.50, 8.34 -> 8.23, 6.47 -> 6.17; up to 660 and less the same within 1%.  The line: with
+// all of the mixed walk's queries by length first the heightfield's up to 660 l_ref took 3.66 ms against
+// 3.61 by place; up to 330, 3.80 against 3.28; up to 55, 0.92 against 0.67.)
 #define SG_FAR_LREF 768.f
 #define SG_FAR_CLASSES 16
 #define SG_FAR_CELLS 1024
@@ -745,7 +748,10 @@ WsLayout ws_layout(int64_t nF, int64_t nq, int sort, bool esc = false, bool orde
 // faster without the start-face order), but lanes holding walks of similar length idle less.
 #define SG_SORT_MIN_BATCH 65536
 // The FP64 walk takes its queries by walk length from this many on: a warp costs the FP64 pipe its
-// longest lane's steps whatever its other lanes do, and the pipe, not the gathers, bounds the walk.
+// longest lane's steps whatever its other lanes do, and the pipe, not the gathers, bounds the walk: on meshes
+// above half of L2 too (a 624,962-face heightfield, 131,000 short walks: 809 us, 1,031 by start face).  Below
+// 65,536 queries, where blocks of one warp give nearly every query a lane, the order itself now costs 0-8% of
+// the call (16,385 queries on a 65,536-face torus 373 us, 356 in input order; 64,000 898 and 838).
 #define SG_SORT64_MIN_BATCH 1024
 // below this many queries the automatic kernel choice walks one thread per query
 #define SG_SMALL_BATCH 65536
