@@ -207,7 +207,8 @@ typedef struct sg_mesh_info {
 } sg_mesh_info;
 
 /* Fills `info`.  After sg_mesh_update_vertices it reads the current l_ref and degenerate
- * count back from the device (a synchronous copy that waits for the update). */
+ * count back from the device (synchronous: it waits for the device, so for an update on any
+ * stream). */
 sg_status sg_mesh_get_info(const sg_mesh *m, sg_mesh_info *info);
 
 /*

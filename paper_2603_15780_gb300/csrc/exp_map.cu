@@ -1029,7 +1029,9 @@ sg_status sg_mesh_get_info(const sg_mesh *m, sg_mesh_info *info) {
         std::vector<int> nd(m->n_mesh);
         double ls = 0.0;
         unsigned long long ne = 0;
-        if (cudaMemcpy(nd.data(), m->d_ndegen, sizeof(int) * nd.size(), cudaMemcpyDeviceToHost) != cudaSuccess ||
+        // (the update may be on a non-blocking stream, for which a copy on the default stream does not wait)
+        if (cudaDeviceSynchronize() != cudaSuccess ||
+            cudaMemcpy(nd.data(), m->d_ndegen, sizeof(int) * nd.size(), cudaMemcpyDeviceToHost) != cudaSuccess ||
             cudaMemcpy(&ls, m->d_lsum, sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess ||
             cudaMemcpy(&ne, m->d_ecount, sizeof(ne), cudaMemcpyDeviceToHost) != cudaSuccess)
             return SG_ERR_CUDA;

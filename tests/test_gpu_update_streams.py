@@ -136,3 +136,20 @@ def test_walks_on_two_streams_after_one_update():
             for o in out:
                 for k in KEYS if kind != "gfd" else ("grad_v", "grad_p", "status"):
                     assert torch.equal(o[k].view(torch.uint8), ref[k].view(torch.uint8)), (kind, k)
+
+
+def test_mesh_info_waits_for_an_update_on_another_stream():
+    torch, sg, mesh, args, start, move = _setup(2000, level=6)
+    made = {id(V): sg.Mesh(V.cpu().numpy(), mesh.F).info().l_ref_mean for V in (start, move)}
+    flat = torch.zeros_like(start)
+    s = torch.cuda.Stream()
+    mesh.update_vertices(start)
+    torch.cuda.synchronize()
+    for V in (move, start, move):
+        with torch.cuda.stream(s):
+            for _ in range(20):                      # enough work ahead of the last update
+                mesh.update_vertices(flat)
+            mesh.update_vertices(V)
+        info = mesh.info()
+        assert info.n_degenerate == 0
+        assert abs(info.l_ref_mean - made[id(V)]) <= 1e-12 * made[id(V)]
