@@ -161,13 +161,21 @@ def _torch():
     return _torch_module
 
 
-def _raw_stream(stream):
-    """cudaStream_t of `stream`, or of torch's current stream (without building a Stream object: two
-    microseconds of each call)."""
-    if stream is not None:
-        return stream.cuda_stream
+def _raw_stream():
+    """cudaStream_t of torch's current stream (without building a Stream object: two microseconds of each
+    call)."""
     torch = _torch()
     return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+
+
+def _on_stream(call, args):
+    """`call` again, with its arguments `args` (its locals() on entry), with the stream among them as
+    torch's current stream: the copies of inputs, the cleared gradients and the scratch that the call makes
+    then belong to that stream, in order with its kernels, and are not handed out again before those ran."""
+    stream = args.pop("stream")
+    args.update(args.pop("opt_kw", {}))
+    with _torch().cuda.stream(stream):
+        return call(**args)
 
 
 def _ptr(t):
@@ -248,10 +256,13 @@ class Mesh:
         torch's current stream).  Returns the device copy of V that the call read; it is
         recorded on the stream, so the caching allocator does not reuse it before the update ran."""
         torch = _torch()
+        if stream is not None:
+            with torch.cuda.stream(stream):
+                return self.update_vertices(V)
         Vd = _dev(V, torch.float32, (-1, 3))
         if Vd.shape[0] != self.n_vertices:
             raise SgError(f"update_vertices: expected {self.n_vertices} vertices, got {Vd.shape[0]}")
-        s = stream if stream is not None else torch.cuda.current_stream()
+        s = torch.cuda.current_stream()
         _check(lib().sg_mesh_update_vertices(self._h, _ptr(Vd), C.c_void_p(s.cuda_stream)),
                "sg_mesh_update_vertices")
         Vd.record_stream(s)
@@ -288,6 +299,8 @@ def exp_map(mesh: Mesh, face, bary, v, w=None, length=None, mesh_id=None, *, wan
     ncross, hash).  `opts` (or keyword overrides such as kernel=KERNEL_PLAIN, sort=0,
     fp64_escalate=0, block=128) map to sg_opts.  `order`: an int32 [nq] CUDA tensor that receives
     the order the queries were walked in (sg_opts.order), for exp_map_backward(order=...)."""
+    if stream is not None:
+        return _on_stream(exp_map, locals())
     torch = _torch()
     face = _dev(face, torch.int32)
     nq = face.numel()
@@ -322,7 +335,7 @@ def exp_map(mesh: Mesh, face, bary, v, w=None, length=None, mesh_id=None, *, wan
     if workspace is not None:
         o.workspace = workspace.data_ptr()
         o.workspace_bytes = workspace.numel()
-    s = _raw_stream(stream)
+    s = _raw_stream()
     rc = lib().sg_exp_map(mesh.handle, nq, _ptr(mesh_id), _ptr(face), _ptr(bary), _ptr(v), _ptr(length), nw,
                           _ptr(w), _ptr(out["face"]), _ptr(out["bary"]), _ptr(out["pos"]), _ptr(out["dir"]),
                           _ptr(out.get("w")), _ptr(out["status"]), _ptr(out.get("ncross")),
@@ -340,6 +353,8 @@ def exp_map_trace(mesh: Mesh, face, bary, v, length=None, mesh_id=None, *, path_
     path_pt [nq, cap, 3] (if want_points), path_len [nq]).  The polyline of query i is
     path_pt[i, :path_len[i]] followed by pos[i] when path_len[i] <= path_cap; path entries
     past path_len are not written (their contents are unspecified)."""
+    if stream is not None:
+        return _on_stream(exp_map_trace, locals())
     torch = _torch()
     face = _dev(face, torch.int32)
     nq = face.numel()
@@ -363,7 +378,7 @@ def exp_map_trace(mesh: Mesh, face, bary, v, length=None, mesh_id=None, *, path_
         workspace = torch.empty(workspace_size(mesh, nq, o), dtype=torch.uint8, device=dev)
     o.workspace = workspace.data_ptr()
     o.workspace_bytes = workspace.numel()
-    s = _raw_stream(stream)
+    s = _raw_stream()
     rc = lib().sg_exp_map_trace(mesh.handle, nq, _ptr(mesh_id), _ptr(face), _ptr(bary), _ptr(v), _ptr(length),
                                 path_cap, _ptr(out["path_face"]), _ptr(out.get("path_pt")), _ptr(out["path_len"]),
                                 _ptr(out["face"]), _ptr(out["bary"]), _ptr(out["pos"]), _ptr(out["dir"]),
@@ -399,6 +414,8 @@ def exp_map_backward(mesh: Mesh, estimator, face, bary, v, end_face, end_bary, e
     point), optional g_bary (end barycentrics), g_dir (end direction), g_w [nq, n_w, 3] (carried
     vectors).  Returns dict(grad_v, grad_p, grad_bary, grad_w (if g_w), grad_V (if requested;
     accumulated into `grad_V` when given), status)."""
+    if stream is not None:
+        return _on_stream(exp_map_backward, locals())
     torch = _torch()
     est = {"ep": EST_EP, "gfd": EST_GFD}.get(estimator, estimator)
     face = _dev(face, torch.int32)
@@ -437,7 +454,7 @@ def exp_map_backward(mesh: Mesh, estimator, face, bary, v, end_face, end_bary, e
                                 device=dev)
     o.workspace = workspace.data_ptr()
     o.workspace_bytes = workspace.numel()
-    s = _raw_stream(stream)
+    s = _raw_stream()
     rc = lib().sg_exp_map_backward(mesh.handle, est, eps_v, eps_p, nq, _ptr(mesh_id), _ptr(face), _ptr(bary),
                                    _ptr(v), _ptr(end_face), _ptr(end_bary), _ptr(end_dir), _ptr(end_status),
                                    _ptr(g_pos), _ptr(g_bary), _ptr(g_dir), n_w, _ptr(g_w if n_w else None),
@@ -453,6 +470,8 @@ def transport_back(mesh: Mesh, face, bary, v, end, u, mesh_id=None, *, opts: Opt
     the geodesics Exp_p(v) back to their start points, the adjoint (= inverse) of the forward
     parallel transport.  `end` is the forward's output dict (face, dir, status).  Returns a
     tensor of u's shape."""
+    if stream is not None:
+        return _on_stream(transport_back, locals())
     torch = _torch()
     face = _dev(face, torch.int32)
     nq = face.numel()
@@ -468,7 +487,7 @@ def transport_back(mesh: Mesh, face, bary, v, end, u, mesh_id=None, *, opts: Opt
     mesh_id = _dev(mesh_id, torch.int32, (nq,))
     out = torch.empty(nq, n_u, 3, device=face.device)
     o = opts if opts is not None else default_opts()
-    s = _raw_stream(stream)
+    s = _raw_stream()
     rc = lib().sg_transport_back(mesh.handle, nq, _ptr(mesh_id), _ptr(face), _ptr(bary), _ptr(v), _ptr(end_face),
                                  _ptr(end_dir), _ptr(end_status), n_u, _ptr(u), _ptr(out), C.byref(o),
                                  s)
@@ -483,6 +502,8 @@ def exp_map_field_steps(mesh: Mesh, face, bary, U, K: int, h: float | None = Non
     one launch; h defaults to 1 / K.  Returns dict(face, bary, pos, dir, status) of the last step,
     with want_steps the per-step records step_face [K+1, nq], step_bary [K+1, nq, 3], step_v [K, nq, 3],
     step_dir [K, nq, 3], step_status [K, nq] (and step_hash [K, nq] with want_hash)."""
+    if stream is not None:
+        return _on_stream(exp_map_field_steps, locals())
     torch = _torch()
     face = _dev(face, torch.int32)
     nq = face.numel()
@@ -505,7 +526,7 @@ def exp_map_field_steps(mesh: Mesh, face, bary, U, K: int, h: float | None = Non
     ws = torch.empty(64, dtype=torch.uint8, device=dev)
     o.workspace = ws.data_ptr()
     o.workspace_bytes = 64
-    s = _raw_stream(stream)
+    s = _raw_stream()
     rc = lib().sg_exp_map_steps(mesh.handle, K, h, _ptr(U), nq, _ptr(mesh_id), _ptr(face), _ptr(bary),
                                 _ptr(out["face"]), _ptr(out["bary"]), _ptr(out["pos"]), _ptr(out["dir"]),
                                 _ptr(out["status"]), _ptr(out.get("step_face")), _ptr(out.get("step_bary")),
@@ -522,6 +543,8 @@ def exp_map_field_steps_backward(mesh: Mesh, estimator, fwd: dict, U, K: int, h:
     """sg_exp_map_steps_backward on the per-step records of exp_map_field_steps.  Returns
     dict(grad_bary [nq, 3] of the start barycentrics, grad_U [n_vertices, 3] (accumulated into
     `grad_U` when given), grad_V (if requested))."""
+    if stream is not None:
+        return _on_stream(exp_map_field_steps_backward, locals())
     torch = _torch()
     est = {"ep": EST_EP, "gfd": EST_GFD}.get(estimator, estimator)
     nq = fwd["face"].numel()
@@ -541,7 +564,7 @@ def exp_map_field_steps_backward(mesh: Mesh, estimator, fwd: dict, U, K: int, h:
     o = opts if opts is not None else default_opts()
     o.workspace = ws.data_ptr()
     o.workspace_bytes = ws.numel()
-    s = _raw_stream(stream)
+    s = _raw_stream()
     rc = lib().sg_exp_map_steps_backward(mesh.handle, est, eps_v, eps_p, K, h, _ptr(U), nq, _ptr(mesh_id),
                                          _ptr(fwd["step_face"]), _ptr(fwd["step_bary"]), _ptr(fwd["step_v"]),
                                          _ptr(fwd["step_dir"]), _ptr(fwd["step_status"]), _ptr(g_pos), _ptr(g_bary),
